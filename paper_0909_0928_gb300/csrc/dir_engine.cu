@@ -389,6 +389,13 @@ static int enqueue_level_start(dir_ctx* c, int lc, char*& cur, char*& oth, cudaS
 }
 
 // Force and smoothing arguments of level lc (buffers, rows and iteration set
+// The stop flag the kernels of level lc look at: none without a stop test, when
+// nothing sets it -- every block of every kernel would begin with a dependent
+// read of it from L2 before its first copy
+static const int* level_stop(const dir_ctx* c, int lc) {
+    return c->p.stop_mode >= 1 ? c->ctl + lc : nullptr;
+}
+
 // by the caller)
 static dirk::ForceArgs level_force_args(const dir_ctx* c, int lc) {
     const int l = c->levels - 1 - lc;
@@ -398,7 +405,7 @@ static dirk::ForceArgs level_force_args(const dir_ctx* c, int lc) {
     fa.M = c->lv[l].M;
     fa.g = g;
     fa.alpha2 = c->p.alpha * c->p.alpha;
-    fa.stop_iter = c->ctl + lc;
+    fa.stop_iter = level_stop(c, lc);
     fa.depth = c->tune_depth[l] ? c->tune_depth[l] : dirk::force_brick_depth(g, c->num_sms);
     // L2 prefetch of the bricks of the block one block per SM ahead (a
     // quarter of a wave of four blocks per SM; measured on 256x256x100
@@ -416,7 +423,7 @@ static dirk::SmoothArgs level_smooth_args(const dir_ctx* c, int lc) {
     sa.g = c->lv[l].g;
     sa.ncomp = 3;
     sa.taps = c->taps;
-    sa.stop_iter = c->ctl + lc;
+    sa.stop_iter = level_stop(c, lc);
     sa.err = c->derr;
     sa.in_type = c->field_type;
     sa.out_type = c->field_type;
@@ -486,7 +493,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                     ua.g = g;
                     ua.taps = c->taps;
                     ua.red = c->red + 3 * (size_t)row;
-                    ua.stop_iter = c->ctl + lc;
+                    ua.stop_iter = level_stop(c, lc);
                     ua.iter = it;
                     ua.err = c->derr;
                     ua.corr = c->corr ? c->corr + 4 * (size_t)row : nullptr;
