@@ -28,6 +28,8 @@ struct Taps {
     double w[17];   // w[t + R] for t = -R..R (normalised)
     float wf[17];   // the same taps rounded for the single-precision path, with
                     // their exact sum kept at 1 (see make_taps in the engine)
+    float2 wp[5];   // wf[0 .. min(R, 4)] on both lanes of a packed pair, so that a
+                    // packed multiply-add can take its tap from the parameter bank
 };
 
 template <typename Real>
@@ -162,38 +164,55 @@ __device__ __forceinline__ Real trilinear(const T* __restrict__ I, const Grid3& 
 // production path: 32 partials of a few voxels each); across warps and blocks
 // they are added in double (the global MSE / convergence reduction).  Every
 // thread of the block must call it.
+//
+// In a warp the three values travel together: after the first two exchanges
+// each 8-lane group holds one of them, so that six shuffles do what fifteen
+// would.  Across the warps lane 8 c + w takes value c of warp w, which needs
+// log2(warps) double additions instead of fifteen (double precision runs at
+// 1/64 of the single-precision rate here, and the block's last warp is alone).
 template <int NT, typename Real>
 __device__ __forceinline__ void block_reduce3_atomic(Real a, Real b, Real c, double* out) {
+    constexpr int NW = NT / 32;
     static_assert(NT % 32 == 0, "block size must be whole warps");
-    __shared__ double red_s[3][NT / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
+    __shared__ Real red_s[3][NW];
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int lane = tid & 31, warp = tid >> 5;
-    if (lane == 0) {
-        red_s[0][warp] = (double)a;
-        red_s[1][warp] = (double)b;
-        red_s[2][warp] = (double)c;
+    {
+        const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
+        Real keep = hi ? c : a;
+        keep += __shfl_xor_sync(0xffffffffu, hi ? a : c, 16);
+        b += __shfl_xor_sync(0xffffffffu, b, 16);
+        const Real send = odd ? keep : b;
+        keep = odd ? b : keep;
+        keep += __shfl_xor_sync(0xffffffffu, send, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+        // lanes 0-7: a, 8-15: b, 16-23: c (24-31: b again)
+        if ((lane & 7) == 0 && lane < 24) red_s[lane >> 3][warp] = keep;
     }
     __syncthreads();
     if (warp == 0) {
-        double da = lane < NT / 32 ? red_s[0][lane] : 0.0;
-        double db = lane < NT / 32 ? red_s[1][lane] : 0.0;
-        double dc = lane < NT / 32 ? red_s[2][lane] : 0.0;
+        if constexpr (NW <= 8) {
+            const int v = lane >> 3, w = lane & 7;
+            double d = (v < 3 && w < NW) ? (double)red_s[v < 3 ? v : 0][w < NW ? w : 0] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            da += __shfl_down_sync(0xffffffffu, da, o);
-            db += __shfl_down_sync(0xffffffffu, db, o);
-            dc += __shfl_down_sync(0xffffffffu, dc, o);
-        }
-        if (lane == 0) {
-            atomicAdd(out + 0, da);
-            atomicAdd(out + 1, db);
-            atomicAdd(out + 2, dc);
+            for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (w == 0 && v < 3) atomicAdd(out + v, d);
+        } else {
+            double da = lane < NW ? (double)red_s[0][lane] : 0.0;
+            double db = lane < NW ? (double)red_s[1][lane] : 0.0;
+            double dc = lane < NW ? (double)red_s[2][lane] : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                da += __shfl_down_sync(0xffffffffu, da, o);
+                db += __shfl_down_sync(0xffffffffu, db, o);
+                dc += __shfl_down_sync(0xffffffffu, dc, o);
+            }
+            if (lane == 0) {
+                atomicAdd(out + 0, da);
+                atomicAdd(out + 1, db);
+                atomicAdd(out + 2, dc);
+            }
         }
     }
 }
@@ -365,6 +384,15 @@ struct BlockPos {
     __device__ __forceinline__ static BlockPos of_grid() {
         return {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                 (int)gridDim.x,  (int)gridDim.y,  (int)gridDim.z};
+    }
+    // the block n positions later (x fastest); false past the end.  32-bit
+    // unsigned divisions: 64-bit ones cost a few hundred instructions here.
+    __device__ __forceinline__ bool ahead(int n, BlockPos& o) const {
+        const unsigned ux = (unsigned)x + (unsigned)n;
+        const unsigned uy = (unsigned)y + ux / (unsigned)gx;
+        const unsigned uz = (unsigned)z + uy / (unsigned)gy;
+        o = {(int)(ux % (unsigned)gx), (int)(uy % (unsigned)gy), (int)uz, gx, gy, gz};
+        return uz < (unsigned)gz;
     }
 };
 

@@ -94,6 +94,7 @@ bool make_taps(double sigma, dirk::Taps* t) {
             }
         }
     }
+    for (int k = 0; k < 5; ++k) t->wp[k] = k <= R ? make_float2(t->wf[k], t->wf[k]) : make_float2(0.0f, 0.0f);
     return true;
 }
 
@@ -388,7 +389,6 @@ static int enqueue_level_start(dir_ctx* c, int lc, char*& cur, char*& oth, cudaS
     return DIR_OK;
 }
 
-// Force and smoothing arguments of level lc (buffers, rows and iteration set
 // The stop flag the kernels of level lc look at: none without a stop test, when
 // nothing sets it -- every block of every kernel would begin with a dependent
 // read of it from L2 before its first copy
@@ -396,6 +396,7 @@ static const int* level_stop(const dir_ctx* c, int lc) {
     return c->p.stop_mode >= 1 ? c->ctl + lc : nullptr;
 }
 
+// Force and smoothing arguments of level lc (buffers, rows and iteration set
 // by the caller)
 static dirk::ForceArgs level_force_args(const dir_ctx* c, int lc) {
     const int l = c->levels - 1 - lc;

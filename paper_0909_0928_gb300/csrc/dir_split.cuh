@@ -34,8 +34,11 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "dir_force_gm.cuh"
 #include "dir_force_kernel.cuh"
+#include "dir_pair.cuh"
 #include "dir_smooth2.cuh"
 #include "dir_stencil.cuh"
 
@@ -69,8 +72,8 @@ __device__ __forceinline__ void zs_block(const CUtensorMap* tmap, const CUtensor
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     float* tb = reinterpret_cast<float*>(base);                      // [3][NPZ][FTY][FTX]
-    const TI* sb = reinterpret_cast<const TI*>(base + F::OFF_S);     // [FTZ+2][FZSH][FSW]
-    const TI* mb = reinterpret_cast<const TI*>(base + F::OFF_M);
+    TI* sb = reinterpret_cast<TI*>(base + F::OFF_S);                 // [FTZ+2][FZSH][FSW]
+    TI* mb = reinterpret_cast<TI*>(base + F::OFF_M);
     uint64_t* bar = reinterpret_cast<uint64_t*>(base + F::OFF_BAR);
     const Grid3 g = a.g;
     const TI* __restrict__ M = static_cast<const TI*>(a.M);
@@ -93,114 +96,106 @@ __device__ __forceinline__ void zs_block(const CUtensorMap* tmap, const CUtensor
         pdl_wait();
         // planes outside the volume arrive zero-filled; replicated below
         tma_load_4d(base, tmap, bx0, by0, bz0 - R, 0, bar);
-        if (a.pf_stride > 0) {  // the block pf_stride positions ahead: its boxes into L2
-            const long long gx = bp.gx, gy = bp.gy;
-            const long long b = bp.x + gx * (bp.y + gy * (long long)bp.z) +
-                                a.pf_stride;
-            if (b < gx * gy * bp.gz) {
-                const int px = (int)(b % gx) * FTX, py = (int)((b / gx) % gy) * FTY;
-                const int pz = (int)(bp.gz - 1 - b / (gx * gy)) * FTZ;
-                tma_prefetch_4d(tmap, px, py, pz - R, 0);
-                tma_prefetch_4d(smap, px - FBX, py - 1, pz - 1, 0);
-                tma_prefetch_4d(mmap, px - FBX, py - 1, pz - 1, 0);
-            }
+        BlockPos nb;
+        if (a.pf_stride > 0 && bp.ahead(a.pf_stride, nb)) {  // that block's boxes into L2
+            const int px = nb.x * FTX, py = nb.y * FTY, pz = (bp.gz - 1 - nb.z) * FTZ;
+            tma_prefetch_4d(tmap, px, py, pz - R, 0);
+            tma_prefetch_4d(smap, px - FBX, py - 1, pz - 1, 0);
+            tma_prefetch_4d(mmap, px - FBX, py - 1, pz - 1, 0);
         }
     }
     pdl_wait();  // every thread: v is written below, which the kernel before reads
     __syncthreads();
-    bool ok = true;
-    if (tid == 0) ok = mbar_wait_bounded(bar, 0, kWaitLimitNs);
-    if (__syncthreads_or(!ok)) {
-        if (tid == 0 && a.err) atomicOr(a.err, kErrTmaTimeout);
-        return;
-    }
-    (void)mbar_try_wait(bar, 0);
+    // every thread waits for the copies itself (bounded); one that gave up
+    // flags the error and goes on over whatever the box holds
+    if (!mbar_wait_bounded(bar, 0, kWaitLimitNs) && a.err) atomicOr(a.err, kErrTmaTimeout);
 
     const int x = bx0 + tx, y = by0 + ty;
-    const bool col_valid = (x < g.nx) && (y < g.ny);
-    float sd2 = 0.0f, sdu = 0.0f, su = 0.0f;
+    PairSums sums;
     CorrSums<float> corr_s;  // with a.corr: the correlation sums
-    if (col_valid) {
-        // z pass of the Gaussian down this thread's column (only this thread
-        // reads or writes it, so no barrier): u[c][k] at z = bz0 + k
-        float w[R + 1];
-#pragma unroll
-        for (int t = 0; t <= R; ++t) w[t] = taps.wf[t];
+    if (x < g.nx && y < g.ny) {
+        // Down this thread's own column: only it reads or writes the column of
+        // t, and the S (M) column outside planes 1 .. FTZ of the box, so
+        // nothing below needs a barrier
         float* tcol = tb + tid;  // plane j of component c at tcol[(c * NPZ + j) * FNT]
+        constexpr int SP = FZSH * FSW;  // elements per plane of an image box
+        const int sx = x - (bx0 - FBX), sy = ty + 1;
+        TI* scol = sb + sy * FSW + sx;
+        TI* mcol = mb + sy * FSW + sx;
         const int zlo = bz0 - R;
         if (zlo < 0 || zlo + NPZ > g.nz) {  // replicate the edge planes into the zero fill
-            const int jlo = max(0, -zlo), jhi = min(NPZ - 1, g.nz - 1 - zlo);
-            for (int c = 0; c < 3; ++c) {
-                float* tc = tcol + c * NPZ * FNT;
-                const float lo = tc[jlo * FNT], hi = tc[jhi * FNT];
-                for (int j = 0; j < jlo; ++j) tc[j * FNT] = lo;
-                for (int j = jhi + 1; j < NPZ; ++j) tc[j * FNT] = hi;
-            }
+            for (int c = 0; c < 3; ++c)
+                replicate_planes(tcol + c * NPZ * FNT, FNT, NPZ, max(0, -zlo),
+                                 min(NPZ - 1, g.nz - 1 - zlo));
+            const int jlo = bz0 == 0 ? 1 : 0, jhi = min(FTZ + 1, g.nz - bz0);
+            replicate_planes(scol, SP, FTZ + 2, jlo, jhi);
+            if (V == 1) replicate_planes(mcol, SP, FTZ + 2, jlo, jhi);
         }
-        // u overwrites t in place (planes R .. R + FTZ - 1 of the column),
-        // which keeps the force loop's registers those of force_tma_kernel
+        constexpr int H = FTZ > 1 ? FTZ / 2 : 1;  // pairs; FTZ = 1: both lanes the one voxel
+        f32x2 up[3][H];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float cv[NPZ];
-#pragma unroll
-            for (int j = 0; j < NPZ; ++j) cv[j] = tcol[(c * NPZ + j) * FNT];
-#pragma unroll
-            for (int k = 0; k < FTZ; ++k) {
-                float acc = 0.0f;
-#pragma unroll
-                for (int t = 0; t < 2 * R + 1; ++t) acc = fmaf(w[t <= R ? t : 2 * R - t], cv[k + t], acc);
-                tcol[(c * NPZ + R + k) * FNT] = acc;
-            }
-        }
+        for (int c = 0; c < 3; ++c)
+            pair_zpass<R, FTZ, H>(tcol + c * NPZ * FNT, FNT, taps, up[c]);
 
-        const int xc = x, yc = y;
-        const int sx = xc - (bx0 - FBX), sxm = max(xc - 1, 0) - (bx0 - FBX);
-        const int sxp = min(xc + 1, g.nx - 1) - (bx0 - FBX);
-        const int sy = yc - (by0 - 1), sym = max(yc - 1, 0) - (by0 - 1);
-        const int syp = min(yc + 1, g.ny - 1) - (by0 - 1);
-        const Interp ip(g);
-        const int cs = (int)g.cs;
+        // x and y neighbours in the box, clamped to the volume
+        const int dxm = x > 0 ? -1 : 0, dxp = x < g.nx - 1 ? 1 : 0;
+        const int dym = y > 0 ? -FSW : 0, dyp = y < g.ny - 1 ? FSW : 0;
+        const PairInterp<TI> ip(g, x, y, bz0);
+        float* __restrict__ vx = v;
+        float* __restrict__ vy = v + g.cs;
+        float* __restrict__ vz = v + 2 * g.cs;
+        const uint32_t o0 = 4u * (uint32_t)offs(g, x, y, bz0), pl = 4u * (uint32_t)g.plane;
+        const f32x2 half = f2_dup(0.5f);
+        auto pairs = [&](auto whole) {  // whole: every plane of the brick lies in the volume
 #pragma unroll
-        for (int k = 0; k < FTZ; ++k) {
-            const int z = bz0 + k;
-            if (z < g.nz) {
-                const int pc = k + 1;
-                const int pm = max(z - 1, 0) - (bz0 - 1), pp = min(z + 1, g.nz - 1) - (bz0 - 1);
-                const TI* Sc = sb + pc * (FZSH * FSW);
-                const float s0 = (float)Sc[sy * FSW + sx];
-                const float gsx = 0.5f * ((float)Sc[sy * FSW + sxp] - (float)Sc[sy * FSW + sxm]);
-                const float gsy = 0.5f * ((float)Sc[syp * FSW + sx] - (float)Sc[sym * FSW + sx]);
-                const float gsz = 0.5f * ((float)sb[pp * (FZSH * FSW) + sy * FSW + sx] -
-                                          (float)sb[pm * (FZSH * FSW) + sy * FSW + sx]);
-                const float ux = tcol[(R + k) * FNT], uy = tcol[(NPZ + R + k) * FNT],
-                            uz = tcol[(2 * NPZ + R + k) * FNT];
-                float bm = 0.0f;
-                if (V == 1) {
-                    const TI* Mc = mb + pc * (FZSH * FSW);
-                    const float mx = 0.5f * ((float)Mc[sy * FSW + sxp] - (float)Mc[sy * FSW + sxm]);
-                    const float my = 0.5f * ((float)Mc[syp * FSW + sx] - (float)Mc[sym * FSW + sx]);
-                    const float mz = 0.5f * ((float)mb[pp * (FZSH * FSW) + sy * FSW + sx] -
-                                             (float)mb[pm * (FZSH * FSW) + sy * FSW + sx]);
-                    bm = r_sqrt(mx * mx + my * my + mz * mz);
+            for (int k = 0; k < H; ++k) {
+                constexpr int HB = FTZ > 1 ? H : 0;
+                const int ka = k, kb = k + HB;
+                const bool va = whole || bz0 + ka < g.nz;
+                const bool vb = FTZ > 1 && (whole || bz0 + kb < g.nz);
+                // half the difference of two image values at both voxels
+                auto grad = [&](const TI* col, int dp, int dm) {
+                    const TI* pa = col + (ka + 1) * SP;
+                    const TI* pb = col + (kb + 1) * SP;
+                    return f2_mul(half, f2_sub(f2_pack(img_bits(pa[dp]), img_bits(pb[dp])),
+                                               f2_pack(img_bits(pa[dm]), img_bits(pb[dm]))));
+                };
+                const f32x2 gs[3] = {grad(scol, dxp, dxm), grad(scol, dyp, dym),
+                                     grad(scol, SP, -SP)};
+                f32x2 bm = 0ull;
+                if (V == 1)
+                    bm = f2_norm_yxz(grad(mcol, dxp, dxm), grad(mcol, dyp, dym), grad(mcol, SP, -SP));
+                const f32x2 s0 =
+                    f2_pack(img_bits(scol[(ka + 1) * SP]), img_bits(scol[(kb + 1) * SP]));
+                const f32x2 u[3] = {up[0][k], up[1][k], up[2][k]};
+                const f32x2 d = ip.at(M, ka, kb, u[0], u[1], u[2], s0);  // W - S
+                if (a.corr) {
+                    if (va) corr_s.add(img_value<TI>(f2_lo(s0)), f2_lo(d));
+                    if (vb) corr_s.add(img_value<TI>(f2_hi(s0)), f2_hi(d));
                 }
-                const float d = interp_rel(M, ip, x, ux, y, uy, z, uz, s0);  // W - S
-                if (a.corr) corr_s.add(s0, d);
-                float dx, dy, dz;
-                demons_force<float, V>(d, gsx, gsy, gsz, 0.0f, 0.0f, 0.0f, bm, 0.0f, dx, dy, dz);
-                dx = -dx;
-                dy = -dy;
-                dz = -dz;
-                sd2 += d * d;
-                sdu += r_norm_fast(dx * dx + dy * dy + dz * dz);
-                su += r_norm_fast(ux * ux + uy * uy + uz * uz);
-                const int o = offs(g, x, y, z);
-                v[o] = ux + dx;
-                v[o + cs] = uy + dy;
-                v[o + 2 * cs] = uz + dz;
+                f32x2 dr[3], vn[3];
+                pair_update<V>(d, gs, gs, bm, 0.0f, u, dr, vn);
+                sums.add(d, dr, u, va, vb);
+                if (va) {
+                    const uint32_t o = o0 + ka * pl;
+                    *at_byte(vx, o) = f2_lo(vn[0]);
+                    *at_byte(vy, o) = f2_lo(vn[1]);
+                    *at_byte(vz, o) = f2_lo(vn[2]);
+                }
+                if (vb) {
+                    const uint32_t o = o0 + kb * pl;
+                    *at_byte(vx, o) = f2_hi(vn[0]);
+                    *at_byte(vy, o) = f2_hi(vn[1]);
+                    *at_byte(vz, o) = f2_hi(vn[2]);
+                }
             }
-        }
+        };
+        if (bz0 + FTZ <= g.nz)
+            pairs(std::true_type{});
+        else
+            pairs(std::false_type{});
     }
-    block_reduce3_atomic<FNT, float>(sd2, sdu, su, a.red);
+    block_reduce3_atomic<FNT, float>(sums.d2, sums.du, sums.u, a.red);
     if (a.corr) block_reduce4_atomic<FNT, float>(corr_s, a.corr);
 }
 

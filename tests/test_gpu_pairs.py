@@ -1,0 +1,49 @@
+"""The production iteration kernels against the plain ones at the sizes where
+their tiling can go wrong: single voxels along an axis, one more and one less
+than a tile, a brick or a strip, volumes thinner than the filter, and brick
+depths that do not divide the volume.  Every kernel rounds each voxel as the
+plain-load kernels do, so the fields must be equal, not close.
+"""
+import numpy as np
+import pytest
+
+from phantom.generator import random_volume
+
+pytestmark = pytest.mark.gpu
+
+# (nx, ny, nz): tiles are 32 wide, 8 to 32 rows high, bricks 1 to 8 planes deep
+DIMS = [(1, 1, 1), (2, 2, 2), (5, 3, 1), (1, 40, 6), (40, 1, 9), (31, 33, 7), (32, 8, 4),
+        (33, 9, 13), (64, 32, 25), (65, 31, 6), (97, 43, 17), (129, 64, 12), (36, 200, 5)]
+
+
+def _run(dl, S, M, dims, variant, i16, **kw):
+    p = dl.dir_params_default(levels=1, iters=[4], alpha=0.7, **kw)
+    ctx = dl.dir_create(S, M, dims, (1.0, 1.0, 1.0), dl.DIR_I16 if i16 else dl.DIR_F32, False,
+                        variant, p)
+    try:
+        dl.dir_register(ctx)
+        u = np.empty((3,) + dims[::-1], np.float32)
+        dl.dir_get_field(ctx, u)
+        return u, dl.dir_get_history(ctx, 4)
+    finally:
+        dl.dir_destroy(ctx)
+
+
+@pytest.mark.parametrize("dims", DIMS, ids=lambda d: "x".join(map(str, d)))
+@pytest.mark.parametrize("i16", [False, True], ids=["f32", "i16"])
+def test_production_kernels_equal_plain(dims, i16):
+    import paper_0909_0928_gb300 as dl
+
+    S = np.round(400.0 * random_volume(dims, 11))
+    M = np.round(400.0 * random_volume(dims, 12))
+    S, M = (a.astype(np.int16 if i16 else np.float32) for a in (S, M))
+    for variant in range(6):
+        # float images for the plain reference: whole numbers, so the same values
+        ref, href = _run(dl, S.astype(np.float32), M.astype(np.float32), dims, variant, False,
+                         plain_kernels=1)
+        for kw in ({}, {"correlation": 1, "pdl": 0}, {"stop_mode": 1, "eps": 0.0}):
+            u, h = _run(dl, S, M, dims, variant, i16, **kw)
+            assert np.array_equal(u, ref, equal_nan=True), (variant, kw, np.abs(u - ref).max())
+            # sums of n positive terms, rounded in FP32 within a thread and a
+            # warp and in FP64 beyond: at most 8 voxels and 32 threads deep
+            np.testing.assert_allclose(h, href, rtol=64 * 2.0 ** -24)
