@@ -244,19 +244,24 @@ static int record(dir_ctx* c, cudaEvent_t e, cudaStream_t s, bool capturing) {
 }
 
 // Issues the whole registration on stream s (captured or direct).
-// Programmatic dependent launch of a level's iteration kernels, above 2^18
-// voxels: a kernel's blocks set up and copy the static images while the one
-// before drains its last wave (they start only once all its blocks have).
-// Measured per level on the 256x256x100 pyramid: 128x128x50 passive 17.96 ->
-// 16.7 us per iteration, 256x256x100 94.15 -> 93.48 us (Eq. 2: 103.8 ->
-// 102.0), but the 64x64x25 level slower (7.19 -> 7.28 us; Eq. 6 18.1 -> 19.7).
+// Programmatic dependent launch of a level's iteration kernels, on levels of
+// 2^19 to 2^20 voxels: a kernel's blocks set up and copy the static images
+// while the one before drains its last wave (they start only once all its
+// blocks have). It pays where a kernel is one or two waves long. Measured per
+// iteration, plain -> dependent, passive / active: 128x128x40 14.66 -> 14.03 /
+// 17.98 -> 17.74 us, 128x128x50 14.84 -> 14.38 / 19.96 -> 19.59, 160x160x40
+// 18.24 -> 18.07 / 22.17 -> 21.27; below, 96x96x48 11.70 -> 12.29 / 14.08 ->
+// 15.56; above, where the early blocks only take memory and slots from the
+// kernel that still runs, 160x160x50 21.22 -> 23.48 / 24.64 -> 25.53,
+// 193x171x87 45.85 -> 46.74 / 59.63 -> 61.32, 256x256x100 72.98 -> 75.43 /
+// 106.97 -> 107.25 (Eq. 6 124.98 -> 127.76).
 // Not with a stop test (the kernels read the stop flag before they wait), nor
-// with timing events between the kernels.  Split schedule only: the same
-// launches made the force + smoothing kernels slower (Eq. 3: 13.20 -> 13.35 ms
-// per registration, Eq. 6: 17.07 -> 17.27; split passive 8.20 -> 8.04).
+// with timing events between the kernels. Split schedule only: the same
+// launches made the force + smoothing kernels slower.
 static bool level_pdl(const dir_ctx* c, const Grid3& g, bool timed) {
+    const long long n = (long long)g.nx * g.ny * g.nz;
     return c->p.pdl && c->p.stop_mode == 0 && !timed && !c->fp64 && !c->p.plain_kernels &&
-           (long long)g.nx * g.ny * g.nz > (1LL << 18);
+           n >= (1LL << 19) && n <= (1LL << 20);
 }
 
 // The split kernels: FP32 field, float or int16 images, radius 3
@@ -1274,13 +1279,13 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             CK(c, dirk::launch_force(c->variant, false, fa, s, false));
             c->launches += 1;
         }
-        int ty = 0, zc = 0, depth = 0;
-        dirk::group_shapes(c0->variant, grids.data(), n, c0->num_sms, &ty, &zc, &depth);
+        int boxes = 0, zc = 0, depth = 0;
+        dirk::group_shapes(c0->variant, grids.data(), n, c0->num_sms, &boxes, &zc, &depth);
         dirk::XYGroup X;
         dirk::ZSGroup Z;
         dirk::ZDGroup ZD;
         dirk::STGroup ST;
-        X.ty = ty;
+        X.boxes = boxes;
         X.zchunk = zc;
         Z.variant = ZD.variant = ST.variant = c0->variant;
         Z.depth = ZD.depth = ST.depth = depth;
@@ -1317,7 +1322,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             }
         }
         const int img = c0->img_type(l);
-        long long chunk_vox = 0;  // the level of the whole chunk, for the rule of level_pdl
+        long long chunk_vox = 0;  // the level of the whole chunk
         for (int q = 0; q < n; ++q) chunk_vox += (long long)grids[q].nx * grids[q].ny * grids[q].nz;
         const bool pdl = c0->p.pdl && chunk_vox > (1LL << 18);
         for (int it = 1; it < iters; ++it) {

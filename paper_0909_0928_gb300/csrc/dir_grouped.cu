@@ -13,6 +13,7 @@
 #include "dir_launch.h"
 #include "dir_split.cuh"
 #include "dir_split_d.cuh"
+#include "dir_xy.cuh"
 
 namespace dirk {
 
@@ -30,13 +31,20 @@ __device__ __forceinline__ BlockPos group_pos(int lb, int gx, int gy, int gz) {
     return {lb % gx, (lb / gx) % gy, lb / (gx * gy), gx, gy, gz};
 }
 
-template <int TY>
-__global__ void __launch_bounds__(8 * TY)
+__global__ void __launch_bounds__(8 * S2Y)
     smooth_xy_grouped_kernel(const __grid_constant__ XYGroup G) {
     const int b = blockIdx.x;
     const int j = group_job(G.first, G.n, b);
-    sxy_block<FZR, TY>(&G.map[j], G.a[j], G.zchunk,
-                       group_pos(b - G.first[j], G.gx[j], G.gy[j], G.gz[j]));
+    sxy_block<FZR, S2Y>(&G.map[j], G.a[j], G.zchunk,
+                        group_pos(b - G.first[j], G.gx[j], G.gy[j], G.gz[j]));
+}
+
+__global__ void __launch_bounds__(32 * XYWARPS)
+    smooth_xy_strip_grouped_kernel(const __grid_constant__ XYGroup G) {
+    const int b = blockIdx.x;
+    const int j = group_job(G.first, G.n, b);
+    const XYStrips st = {G.boxes, G.gx[j], G.gy[j], G.gz[j]};
+    xy_strip_block(&G.map[j], G.a[j], st, b - G.first[j]);
 }
 
 template <int V, int FTZ, typename TI>
@@ -67,34 +75,28 @@ __global__ void __launch_bounds__(FNT, 4) force_st_grouped_kernel(const __grid_c
                          group_pos(b - G.first[j], G.gx[j], G.gy[j], G.gz[j]));
 }
 
-// x/y kernel shared memory of a tile height
-static int sxy_smem(int ty) { return ty == 32 ? SXYSmem<FZR, 32>::SMEM : SXYSmem<FZR, S2Y>::SMEM; }
-
-void group_shapes(int variant, const Grid3* grids, int n, int num_sms, int* ty, int* zchunk,
+void group_shapes(int variant, const Grid3* grids, int n, int num_sms, int* boxes, int* zchunk,
                   int* depth) {
-    // tile rows: 32 where the group has enough tall tiles to fill the GPU
-    long long tall = 0;
-    for (int j = 0; j < n; ++j)
-        tall += (long long)((grids[j].nx + S2X - 1) / S2X) * ((grids[j].ny + 31) / 32) * 3 *
-                grids[j].nz;
-    *ty = tall >= 8LL * num_sms ? 32 : S2Y;
-    // z chunk: the longest of 4, 2, 1 planes that still gives a wave of blocks
-    static KernelSetup s32, s16;
+    static KernelSetup strips, tiles;
     int per_sm = 1;
-    if (*ty == 32)
-        setup_kernel(s32, smooth_xy_grouped_kernel<32>, sxy_smem(32), 8 * 32, &per_sm);
-    else
-        setup_kernel(s16, smooth_xy_grouped_kernel<S2Y>, sxy_smem(S2Y), 8 * S2Y, &per_sm);
-    const long long slots = (long long)(per_sm < 1 ? 1 : per_sm) * num_sms;
-    *zchunk = 1;
-    for (int c = 4; c > 1; c /= 2) {
-        long long blocks = 0;
-        for (int j = 0; j < n; ++j)
-            blocks += (long long)((grids[j].nx + S2X - 1) / S2X) *
-                      ((grids[j].ny + *ty - 1) / *ty) * 3 * ((grids[j].nz + c - 1) / c);
-        if (blocks >= slots) {
-            *zchunk = c;
-            break;
+    *boxes = *zchunk = 0;
+    if (xy_use_strips(grids, n, num_sms)) {
+        setup_kernel(strips, smooth_xy_strip_grouped_kernel, XYSMEM, 32 * XYWARPS, &per_sm);
+        *boxes = xy_strip_boxes(grids, n, (long long)per_sm * num_sms * XYWARPS);
+    } else {
+        // z chunk: the longest of 4, 2, 1 planes that still gives a wave of blocks
+        setup_kernel(tiles, smooth_xy_grouped_kernel, SXYSmem<FZR, S2Y>::SMEM, 8 * S2Y, &per_sm);
+        const long long slots = (long long)(per_sm < 1 ? 1 : per_sm) * num_sms;
+        *zchunk = 1;
+        for (int c = 4; c > 1; c /= 2) {
+            long long blocks = 0;
+            for (int j = 0; j < n; ++j)
+                blocks += (long long)((grids[j].nx + S2X - 1) / S2X) *
+                          ((grids[j].ny + S2Y - 1) / S2Y) * 3 * ((grids[j].nz + c - 1) / c);
+            if (blocks >= slots) {
+                *zchunk = c;
+                break;
+            }
         }
     }
     // brick depth: the one-volume rules (force_zs_depth, force_brick_depth) on
@@ -133,19 +135,30 @@ static bool encode4(CUtensorMap* m, CUtensorMapDataType t, const void* p, const 
 }
 
 bool xy_group_add(XYGroup& G, const SmoothArgs& a) {
-    if (G.n >= kGroupMax || (G.ty != 32 && G.ty != S2Y) || G.zchunk < 1 || a.ncomp != 3 ||
+    if (G.n >= kGroupMax || (G.boxes < 2 && G.zchunk < 1) || a.ncomp != 3 ||
         a.in_type != kStoreF32 || a.out_type != kStoreF32 || a.taps.R != FZR)
         return false;
     const int j = G.n;
     if (j == 0) G.first[0] = 0;
-    const int H = G.ty + 2 * FZR, WB = S2Geom<FZR>::WB;  // the plane box of sxy_block
-    const cuuint32_t box[4] = {(cuuint32_t)WB, (cuuint32_t)H, 1u, 1u};
-    if (!encode4(&G.map[j], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.in, a.g, 3, 4, box)) return false;
+    int blocks;
+    if (G.boxes > 0) {
+        if (!make_xy_strip_map(&G.map[j], a.in, a.g)) return false;
+        const XYStrips st = xy_strips(a.g, G.boxes);
+        G.gx[j] = st.tx;
+        G.gy[j] = st.cy;
+        G.gz[j] = st.n;
+        blocks = st.blocks();
+    } else {
+        const int H = S2Y + 2 * FZR, WB = S2Geom<FZR>::WB;  // the plane box of sxy_block
+        const cuuint32_t box[4] = {(cuuint32_t)WB, (cuuint32_t)H, 1u, 1u};
+        if (!encode4(&G.map[j], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.in, a.g, 3, 4, box)) return false;
+        G.gx[j] = (a.g.nx + S2X - 1) / S2X;
+        G.gy[j] = (a.g.ny + S2Y - 1) / S2Y;
+        G.gz[j] = ((a.g.nz + G.zchunk - 1) / G.zchunk) * 3;
+        blocks = G.gx[j] * G.gy[j] * G.gz[j];
+    }
     G.a[j] = a;
-    G.gx[j] = (a.g.nx + S2X - 1) / S2X;
-    G.gy[j] = (a.g.ny + G.ty - 1) / G.ty;
-    G.gz[j] = ((a.g.nz + G.zchunk - 1) / G.zchunk) * 3;
-    G.first[j + 1] = G.first[j] + G.gx[j] * G.gy[j] * G.gz[j];
+    G.first[j + 1] = G.first[j] + blocks;
     G.n = j + 1;
     return true;
 }
@@ -184,19 +197,17 @@ bool zs_group_add(ZSGroup& G, const ForceArgs& a) {
 cudaError_t launch_smooth_xy_grouped(const XYGroup& G, cudaStream_t s, bool pdl) {
     if (G.n < 1 || G.first[G.n] < 1) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)G.first[G.n]);
-    if (G.ty == 32) {
+    if (G.boxes > 0) {
         static KernelSetup st;
-        const cudaError_t e = setup_kernel(st, smooth_xy_grouped_kernel<32>, sxy_smem(32));
+        const cudaError_t e = setup_kernel(st, smooth_xy_strip_grouped_kernel, XYSMEM);
         if (e != cudaSuccess) return e;
-        return launch_ex(smooth_xy_grouped_kernel<32>, grid, dim3(8 * 32), sxy_smem(32), s, pdl, G);
-    } else if (G.ty == S2Y) {
-        static KernelSetup st;
-        const cudaError_t e = setup_kernel(st, smooth_xy_grouped_kernel<S2Y>, sxy_smem(S2Y));
-        if (e != cudaSuccess) return e;
-        return launch_ex(smooth_xy_grouped_kernel<S2Y>, grid, dim3(8 * S2Y), sxy_smem(S2Y), s, pdl,
-                         G);
+        return launch_ex(smooth_xy_strip_grouped_kernel, grid, dim3(32 * XYWARPS), XYSMEM, s, pdl, G);
     }
-    return cudaErrorInvalidValue;
+    constexpr int SMEM = SXYSmem<FZR, S2Y>::SMEM;
+    static KernelSetup st;
+    const cudaError_t e = setup_kernel(st, smooth_xy_grouped_kernel, SMEM);
+    if (e != cudaSuccess) return e;
+    return launch_ex(smooth_xy_grouped_kernel, grid, dim3(8 * S2Y), SMEM, s, pdl, G);
 }
 
 template <int V, int FTZ, typename TI>

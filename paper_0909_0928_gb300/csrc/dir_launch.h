@@ -63,7 +63,8 @@ struct SmoothArgs {
     int* err;            // device error word (kErr* bits)
     int in_type;         // storage of in (kStore*)
     int out_type;        // storage of out
-    int zchunk;          // planes per block; 0 = one wave of resident blocks
+    int zchunk;          // planes per block; 0 = one wave of resident blocks (x/y strips:
+                         // boxes per strip; 0 = the launcher's rule)
     bool pdl = false;    // as ForceArgs::pdl (the x/y kernel)
 };
 // plain = true: the 32 x 8 tile kernel (smooth_kernel) for every storage type
@@ -72,7 +73,7 @@ cudaError_t launch_smooth(bool fp64, const SmoothArgs& a, int num_sms, cudaStrea
                           bool plain = false);
 
 // The x and y passes of the Gaussian alone, plane by plane (single precision,
-// three components, radius 1..4): out = G_y * G_x * in.  With
+// three components, radius 3): out = G_y * G_x * in.  With
 // launch_force_zs, which applies G_z, one smoothing + force iteration.
 bool smooth_xy_supported(const SmoothArgs& a);
 cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s);
@@ -110,10 +111,10 @@ struct XYGroup {
     CUtensorMap map[kGroupMax];  // each job's plane box of v (x/y kernel layout)
     SmoothArgs a[kGroupMax];
     int first[kGroupMax + 1];
-    int gx[kGroupMax], gy[kGroupMax], gz[kGroupMax];
+    int gx[kGroupMax], gy[kGroupMax], gz[kGroupMax];  // strips: tiles, strips along y, strips
     int n = 0;                   // jobs
-    int ty = 0;                  // tile rows, 16 or 32 (all jobs)
-    int zchunk = 0;              // planes per block (all jobs)
+    int boxes = 0;               // strips of this many boxes (dir_xy.cuh), or 0: tiles
+    int zchunk = 0;              // tiles: planes per block
 };
 struct ZSGroup {
     CUtensorMap tmap[kGroupMax], smap[kGroupMax], mmap[kGroupMax];
@@ -125,10 +126,10 @@ struct ZSGroup {
     int variant = 0;             // force law (all jobs)
     int depth = 0;               // brick depth (all jobs)
 };
-// Shapes for a group of jobs with the given level grids: the x/y kernel's tile
-// rows and z chunk, and the z + force kernel's brick depth (the one-volume
+// Shapes for a group of jobs with the given level grids: the x/y kernel's strip
+// length or z chunk, and the z + force kernel's brick depth (the one-volume
 // rules applied to the group's total block count).
-void group_shapes(int variant, const Grid3* grids, int n, int num_sms, int* ty, int* zchunk,
+void group_shapes(int variant, const Grid3* grids, int n, int num_sms, int* boxes, int* zchunk,
                   int* depth);
 // Add a job (its arguments; a.in / a.u its input field) to a group with
 // shapes already set; false if a tensor map cannot be made.

@@ -15,11 +15,14 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "dir_common.cuh"
 #include "dir_launch.h"
 #include "dir_smooth2.cuh"
 #include "dir_split.cuh"
 #include "dir_stencil.cuh"
+#include "dir_xy.cuh"
 
 namespace dirk {
 
@@ -180,17 +183,22 @@ __global__ void __launch_bounds__(8 * TY, 16 / TY * 8)
 }
 
 // ---------------------------------------------------------------------------
-// The x and y passes alone (single precision, three components), for the
-// schedule that runs the z pass inside the force kernel (dir_force_tma.cu):
-// out(x, y, z) = G_y * G_x * in on every plane, plane by plane.  Without a z
-// pass there is no z halo, so a block's z chunk can be as short as the
-// occupancy wants at no extra work, and there is no ring of filtered planes.
-// Same building blocks, layout and order of operations as smooth2_kernel.
+// The x and y passes alone (single precision, three components, radius 3), for
+// the schedule that runs the z pass inside the force kernel: out = G_y * G_x *
+// in on every plane, plane by plane.  Same order of operations as
+// smooth2_kernel, in two forms: warps marching down y (dir_xy.cuh) on levels
+// that fill the GPU with them, and on smaller ones blocks of 32 x 16 tiles
+// (sxy_block), whose shorter chain of dependent steps counts there.
 // ---------------------------------------------------------------------------
-template <int R, int TY>
-__global__ void __launch_bounds__(8 * TY)
+__global__ void __launch_bounds__(32 * XYWARPS)
+    smooth_xy_strip_kernel(const __grid_constant__ CUtensorMap tmap, const SmoothArgs a,
+                           const XYStrips st) {
+    xy_strip_block(&tmap, a, st, blockIdx.x);
+}
+
+__global__ void __launch_bounds__(8 * S2Y)
     smooth_xy_kernel(const __grid_constant__ CUtensorMap tmap, const SmoothArgs a, int zchunk) {
-    sxy_block<R, TY>(&tmap, a, zchunk, BlockPos::of_grid());
+    sxy_block<XYR, S2Y>(&tmap, a, zchunk, BlockPos::of_grid());
 }
 
 // ---------------------------------------------------------------------------
@@ -395,22 +403,20 @@ static cudaError_t launch_s2t(const SmoothArgs& a, int num_sms, cudaStream_t s) 
     return launch_s2<R, S2Y>(a, num_sms, s);
 }
 
-template <int R, int TY>
 static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, cudaStream_t s) {
-    using G = SXYSmem<R, TY>;
+    using G = SXYSmem<XYR, S2Y>;
     CUtensorMap map;
-    if (!make_s2_map<R, TY>(&map, a.in, a.g, a.ncomp)) return cudaErrorInvalidValue;
-    static KernelSetup setup;  // per instantiation
+    if (!make_s2_map<XYR, S2Y>(&map, a.in, a.g, a.ncomp)) return cudaErrorInvalidValue;
+    static KernelSetup setup;
     int per_sm = 1;
-    const cudaError_t e = setup_kernel(setup, smooth_xy_kernel<R, TY>, G::SMEM, 8 * TY, &per_sm);
+    const cudaError_t e = setup_kernel(setup, smooth_xy_kernel, G::SMEM, 8 * S2Y, &per_sm);
     if (e != cudaSuccess) return e;
     // No z halo, so short chunks cost nothing extra: the longest of 4, 2, 1
-    // planes that still gives a wave of resident blocks (the autotuner's choice
-    // on each level of the 256x256x100 pyramid)
+    // planes that still gives a wave of resident blocks
     int zc = a.zchunk;
     if (zc <= 0) {
         const long long bxy =
-            (long long)((a.g.nx + S2X - 1) / S2X) * ((a.g.ny + TY - 1) / TY) * a.ncomp;
+            (long long)((a.g.nx + S2X - 1) / S2X) * ((a.g.ny + S2Y - 1) / S2Y) * a.ncomp;
         const long long slots = (long long)(per_sm < 1 ? 1 : per_sm) * num_sms;
         zc = 1;
         for (int c = 4; c > 1; c /= 2)
@@ -421,8 +427,23 @@ static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, cudaStream_t s) 
     }
     if (zc > a.g.nz) zc = a.g.nz;
     const int chunks = (a.g.nz + zc - 1) / zc;
-    const dim3 grid((a.g.nx + S2X - 1) / S2X, (a.g.ny + TY - 1) / TY, chunks * a.ncomp);
-    return launch_ex(smooth_xy_kernel<R, TY>, grid, dim3(8 * TY, 1, 1), G::SMEM, s, a.pdl, map, a, zc);
+    const dim3 grid((a.g.nx + S2X - 1) / S2X, (a.g.ny + S2Y - 1) / S2Y, chunks * a.ncomp);
+    return launch_ex(smooth_xy_kernel, grid, dim3(8 * S2Y, 1, 1), G::SMEM, s, a.pdl, map, a, zc);
+}
+
+static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, cudaStream_t s) {
+    CUtensorMap map;
+    if (!make_xy_strip_map(&map, a.in, a.g)) return cudaErrorInvalidValue;
+    static KernelSetup setup;
+    int per_sm = 1;
+    const cudaError_t e =
+        setup_kernel(setup, smooth_xy_strip_kernel, XYSMEM, 32 * XYWARPS, &per_sm);
+    if (e != cudaSuccess) return e;
+    const int nb = a.zchunk > 0 ? std::max(2, std::min(a.zchunk, 64))
+                                : xy_strip_boxes(&a.g, 1, per_sm * num_sms * XYWARPS);
+    const XYStrips st = xy_strips(a.g, nb);
+    return launch_ex(smooth_xy_strip_kernel, dim3((unsigned)st.blocks()), dim3(32 * XYWARPS, 1, 1),
+                     XYSMEM, s, a.pdl, map, a, st);
 }
 
 template <typename Real, int R, typename TIN, typename TOUT>
@@ -459,21 +480,13 @@ static cudaError_t launch_types(const SmoothArgs& a, int num_sms, cudaStream_t s
 }
 
 bool smooth_xy_supported(const SmoothArgs& a) {
-    return a.ncomp == 3 && a.in_type == kStoreF32 && a.out_type == kStoreF32 && a.taps.R >= 1 &&
-           a.taps.R <= 4;
+    return a.ncomp == 3 && a.in_type == kStoreF32 && a.out_type == kStoreF32 && a.taps.R == XYR;
 }
 
 cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s) {
     if (!smooth_xy_supported(a)) return cudaErrorInvalidValue;
-    const long long tiles32 = (long long)((a.g.nx + S2X - 1) / S2X) * ((a.g.ny + 31) / 32) * a.ncomp;
-    const bool tall = tiles32 * a.g.nz >= 8LL * num_sms;
-    switch (a.taps.R) {
-        case 1: return tall ? launch_sxy<1, 32>(a, num_sms, s) : launch_sxy<1, S2Y>(a, num_sms, s);
-        case 2: return tall ? launch_sxy<2, 32>(a, num_sms, s) : launch_sxy<2, S2Y>(a, num_sms, s);
-        case 3: return tall ? launch_sxy<3, 32>(a, num_sms, s) : launch_sxy<3, S2Y>(a, num_sms, s);
-        case 4: return tall ? launch_sxy<4, 32>(a, num_sms, s) : launch_sxy<4, S2Y>(a, num_sms, s);
-        default: return cudaErrorInvalidValue;
-    }
+    return xy_use_strips(&a.g, 1, num_sms) ? launch_xy_strips(a, num_sms, s)
+                                           : launch_sxy(a, num_sms, s);
 }
 
 cudaError_t launch_smooth(bool fp64, const SmoothArgs& a, int num_sms, cudaStream_t s,
