@@ -114,8 +114,8 @@ typedef struct {
                                     field, float or int16 images, sigma with radius 3, any
                                     stop_mode), every level.  4: as 3, but Eqs. (3)-(6) split
                                     once more after the difference image: a z-pass kernel
-                                    writes u and D = W - S once per voxel (Eq. 6: both warped
-                                    differences) to a scratch of 4 (Eq. 6: 5) floats per voxel
+                                    writes D = W - S once per voxel (Eq. 6: both warped
+                                    differences) to a scratch of 1 (Eq. 6: 2) floats per voxel
                                     of the level, and a stencil kernel forms the force from
                                     them, instead of interpolating W on every brick's halo.
                                     2 (default): as 4 where it applies.  dir_register_noalloc

@@ -130,7 +130,7 @@ struct dir_ctx {
     char* img_pool = nullptr;
     char* A = nullptr;
     char* B = nullptr;
-    char* C = nullptr;     // Eqs. 3-6 split with the difference image: u and D of a level
+    char* C = nullptr;     // Eqs. 3-6 split with the difference image: D of a level
     size_t C_bytes = 0;
     double* red = nullptr;
     double* corr = nullptr;   // 4 sums per iteration of the correlation coefficient, or null
@@ -278,7 +278,7 @@ static bool level_split_ok(const dir_ctx* c, int l) {
 // finest level, the force + smoothing kernels (schedule 0), active: 125.4 us
 // against 169.7 and 148.6 on the finest level, 21.7 against 27.8 on
 // 128x128x50, 10.2 against 10.5 on 64x64x25; Eq. 6: 170.8 against 229.1 and
-// 207.8, 36.6 against 45.4, 16.8 against 17.8.  It needs the u + D scratch
+// 207.8, 36.6 against 45.4, 16.8 against 17.8.  It needs the D scratch
 // (dir_ctx::C), allocated for the levels that run it; without one
 // (dir_register_noalloc) a level runs what the rules below give.
 static bool level_wants_d(const dir_ctx* c, int l) {
@@ -293,7 +293,20 @@ static bool level_wants_d(const dir_ctx* c, int l) {
 constexpr int kZdMaxDepth = 4;
 
 static size_t level_d_bytes(const dir_ctx* c, int l) {
-    return (size_t)dirk::force_d_planes(c->variant) * (size_t)c->lv[l].g.cs * sizeof(float);
+    return (size_t)dirk::force_d_planes(c->variant, c->lv[l].g) * (size_t)c->lv[l].g.cs *
+           sizeof(float);
+}
+
+// The scratch of schedule 3 into the arguments of its two kernels: D, Eq. 6's d,
+// then u where the z + D kernel writes it (else both read t from their u)
+static void d_scratch(const dir_ctx* c, const Grid3& g, bool writes_u, dirk::ForceArgs& za,
+                      dirk::ForceArgs& ta) {
+    const size_t plane = (size_t)g.cs * sizeof(float);
+    const bool ic = c->variant == DIR_INVERSE_CONSISTENT;
+    za.dbuf = ta.dbuf = c->C;
+    za.dbuf2 = ta.dbuf2 = ic ? c->C + plane : nullptr;
+    if (writes_u) za.v = c->C + (ic ? 2 : 1) * plane;
+    if (writes_u) ta.u = za.v;
 }
 
 // Iteration schedule of pyramid level l: 0 force + smoothing kernels, 1 fused
@@ -531,8 +544,8 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
         if ((sched == 2 || sched == 3) && n > 0) {
             // iteration 0 from u; iteration k > 0: t = G_y G_x v (xy kernel), then
             // v = u - dr(u) with u = G_z t (force kernel; schedule 3: the z + D
-            // kernel writes u and D to the scratch, the stencil force kernel
-            // reads them); then u = G v of the last iteration run
+            // kernel writes D to the scratch, the stencil force kernel reads it);
+            // then u = G v of the last iteration run
             char* vbuf = oth;
             char* tbuf = cur;
             dirk::SmoothArgs xa = sa;
@@ -542,7 +555,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
             // brick depths: of the z + force kernel (tuned or its own rule), and
             // of the plain force pass of iteration 0
             const int zs_depth = c->tune_depth[l] ? c->tune_depth[l]
-                                 : sched == 3 ? dirk::force_d_depth(g, c->num_sms)
+                                 : sched == 3 ? dirk::force_d_depth(c->variant, g, c->num_sms)
                                               : dirk::force_zs_depth(c->variant, g, c->num_sms);
             const int first_depth = dirk::force_brick_depth(g, c->num_sms);
             const bool pdl = level_pdl(c, g, timed);
@@ -568,15 +581,9 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                     fa.pdl = pdl;
                     if (sched == 3) {
                         dirk::ForceArgs za = fa, ta = fa;
-                        char* dpl = c->C + 3 * (size_t)g.cs * sizeof(float);
                         za.depth = std::min(zs_depth, kZdMaxDepth);
-                        za.u = tbuf;
-                        za.v = c->C;
-                        za.dbuf = ta.dbuf = dpl;
-                        za.dbuf2 = ta.dbuf2 =
-                            c->variant == DIR_INVERSE_CONSISTENT ? dpl + (size_t)g.cs * sizeof(float)
-                                                                 : nullptr;
-                        ta.u = c->C;
+                        za.u = ta.u = tbuf;
+                        d_scratch(c, g, dirk::force_d_writes_u(g), za, ta);
                         CK(c, dirk::launch_force_d(c->variant, za, ta, c->taps, s));
                         c->launches += 3;
                     } else {
@@ -852,7 +859,7 @@ int dir_create(dir_ctx** out, const void* static_img, const void* moving_img, co
         c->lv[l].S = c->img_pool + img_off[l][0];
         c->lv[l].M = c->img_pool + img_off[l][1];
     }
-    // the u + D scratch of schedule 3, for the largest level that runs it
+    // the D scratch of schedule 3, for the largest level that runs it
     for (int l = 0; l < c->levels; ++l)
         if (p.iters[c->levels - 1 - l] > 0 && level_wants_d(c, l))
             c->C_bytes = std::max(c->C_bytes, level_d_bytes(c, l));
@@ -1258,7 +1265,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             grids[q] = c->lv[l].g;
         }
         if (iters == 0) continue;
-        // Eqs. 3-6 where every job has its u + D scratch: the split after the
+        // Eqs. 3-6 where every job has its D scratch: the split after the
         // difference image, as each job's own registration would run it
         bool dform = c0->variant >= 2;
         for (int q = 0; q < n; ++q) {
@@ -1279,6 +1286,8 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             CK(c, dirk::launch_force(c->variant, false, fa, s, false));
             c->launches += 1;
         }
+        long long chunk_vox = 0;  // the level of the whole chunk
+        for (int q = 0; q < n; ++q) chunk_vox += (long long)grids[q].nx * grids[q].ny * grids[q].nz;
         int boxes = 0, zc = 0, depth = 0;
         dirk::group_shapes(c0->variant, grids.data(), n, c0->num_sms, &boxes, &zc, &depth);
         dirk::XYGroup X;
@@ -1286,10 +1295,12 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
         dirk::ZDGroup ZD;
         dirk::STGroup ST;
         X.boxes = boxes;
+        // the rule of one volume on the whole chunk (each job then has room for u)
+        ZD.writes_u = ST.writes_u = dirk::force_d_writes_u(chunk_vox);
         X.zchunk = zc;
         Z.variant = ZD.variant = ST.variant = c0->variant;
         Z.depth = ZD.depth = ST.depth = depth;
-        Z.taps = ZD.taps = c0->taps;
+        Z.taps = ZD.taps = ST.taps = c0->taps;
         for (int q = 0; q < n; ++q) {
             dir_ctx* c = ctxs[jobs[q]];
             dirk::SmoothArgs sa = level_smooth_args(c, lc);
@@ -1305,13 +1316,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             bool added = dirk::xy_group_add(X, sa);
             if (dform) {
                 dirk::ForceArgs za = fa, ta = fa;
-                char* dpl = c->C + 3 * (size_t)grids[q].cs * sizeof(float);
-                za.v = c->C;
-                ta.u = c->C;
-                za.dbuf = ta.dbuf = dpl;
-                za.dbuf2 = ta.dbuf2 = c->variant == DIR_INVERSE_CONSISTENT
-                                          ? dpl + (size_t)grids[q].cs * sizeof(float)
-                                          : nullptr;
+                d_scratch(c, grids[q], ZD.writes_u, za, ta);
                 added = added && dirk::d_group_add(ZD, ST, za, ta);
             } else {
                 added = added && dirk::zs_group_add(Z, fa);
@@ -1322,8 +1327,6 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             }
         }
         const int img = c0->img_type(l);
-        long long chunk_vox = 0;  // the level of the whole chunk
-        for (int q = 0; q < n; ++q) chunk_vox += (long long)grids[q].nx * grids[q].ny * grids[q].nz;
         const bool pdl = c0->p.pdl && chunk_vox > (1LL << 18);
         for (int it = 1; it < iters; ++it) {
             for (int q = 0; q < n; ++q) {
@@ -1573,16 +1576,10 @@ extern "C" int dir_autotune(dir_ctx* c, int reps, int* shapes_out) {
         float best = 1e30f;
         int best_d = 0;
         const int depths[5] = {1, 2, 4, 8, 6};  // 6: the split force kernel only
-        // schedule 3: the z + D and stencil force kernels, u and D in the scratch
+        // schedule 3: the z + D and stencil force kernels, D in the scratch
         dirk::ForceArgs za = fa, ta = fa;
         if (sched == 3) {
-            char* dpl = c->C + 3 * (size_t)g.cs * sizeof(float);
-            za.v = c->C;
-            ta.u = c->C;
-            za.dbuf = ta.dbuf = dpl;
-            za.dbuf2 = ta.dbuf2 = c->variant == DIR_INVERSE_CONSISTENT
-                                      ? dpl + (size_t)g.cs * sizeof(float)
-                                      : nullptr;
+            d_scratch(c, g, dirk::force_d_writes_u(g), za, ta);
         }
         for (int di = 0; di < (sched == 2 ? 5 : 4) && rc == DIR_OK; ++di) {
             const int d = depths[di];

@@ -8,19 +8,19 @@
 
 namespace dirk {
 
-template <int V, int FTZ, typename TI>
-__global__ void __launch_bounds__(FNT, 4)
+template <int V, int FTZ, typename TI, bool UW>
+__global__ void __launch_bounds__(FNT, UW || V == 5 ? 4 : 5)
     force_zd_kernel(const __grid_constant__ CUtensorMap tmap, const ForceArgs a, const Taps taps) {
-    zd_block<V, FTZ, TI>(&tmap, a, taps, BlockPos::of_grid());
+    zd_block<V, FTZ, TI, UW>(&tmap, a, taps, BlockPos::of_grid());
 }
 
-template <int V, int FTZ, typename TI>
-__global__ void __launch_bounds__(FNT, 4)
+template <int V, int FTZ, typename TI, bool UW>
+__global__ void __launch_bounds__(FNT, UW ? 4 : 3)
     force_st_kernel(const __grid_constant__ CUtensorMap dmap,
                     const __grid_constant__ CUtensorMap smap,
-                    const __grid_constant__ CUtensorMap umap,
-                    const __grid_constant__ CUtensorMap emap, const ForceArgs a) {
-    st_block<V, FTZ, TI>(&dmap, &smap, &umap, &emap, a, BlockPos::of_grid());
+                    const __grid_constant__ CUtensorMap tmap,
+                    const __grid_constant__ CUtensorMap emap, const ForceArgs a, const Taps taps) {
+    st_block<V, FTZ, TI, UW>(&dmap, &smap, &tmap, &emap, a, taps, BlockPos::of_grid());
 }
 
 namespace {
@@ -45,59 +45,65 @@ dim3 brick_grid(const Grid3& g, int ftz) {
     return dim3((g.nx + FTX - 1) / FTX, (g.ny + FTY - 1) / FTY, (g.nz + ftz - 1) / ftz);
 }
 
-template <int V, int FTZ, typename TI>
+template <int V, int FTZ, typename TI, bool UW>
 cudaError_t launch_zd(const ForceArgs& a, const Taps& taps, cudaStream_t s) {
     using Z = ZDGeom<FTZ>;
     CUtensorMap tmap;
     if (!map4(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.u, a.g, 3, 4, FTX, FTY, Z::NPZ))
         return cudaErrorInvalidValue;
     static KernelSetup setup;  // per instantiation
-    const cudaError_t e = setup_kernel(setup, force_zd_kernel<V, FTZ, TI>, Z::SMEM);
+    const cudaError_t e = setup_kernel(setup, force_zd_kernel<V, FTZ, TI, UW>, Z::SMEM);
     if (e != cudaSuccess) return e;
-    return launch_ex(force_zd_kernel<V, FTZ, TI>, brick_grid(a.g, FTZ), dim3(FTX, FTY, 1), Z::SMEM,
-                     s, a.pdl, tmap, a, taps);
+    return launch_ex(force_zd_kernel<V, FTZ, TI, UW>, brick_grid(a.g, FTZ), dim3(FTX, FTY, 1),
+                     Z::SMEM, s, a.pdl, tmap, a, taps);
 }
 
-template <int V, int FTZ, typename TI>
-cudaError_t launch_st(const ForceArgs& a, cudaStream_t s) {
-    using F = STGeom<FTZ, V, TI>;
-    CUtensorMap dmap, smap, umap, emap;
+template <int V, int FTZ, typename TI, bool UW>
+cudaError_t launch_st(const ForceArgs& a, const Taps& taps, cudaStream_t s) {
+    using F = STGeom<FTZ, V, TI, UW>;
+    CUtensorMap dmap, smap, tmap, emap;
     if (!map4(&dmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.dbuf, a.g, 1, 4, F::DW, F::DH, F::DD) ||
         !map4(&smap, tma_type<TI>(), a.S, a.g, 1, (int)sizeof(TI), F::FSW, FSH, F::DD) ||
-        !map4(&umap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.u, a.g, 3, 4, FTX, FTY, FTZ))
+        !map4(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.u, a.g, 3, 4, FTX, FTY, F::NPZ))
         return cudaErrorInvalidValue;
     if (F::IC) {
         if (!map4(&emap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.dbuf2, a.g, 1, 4, FTX, FTY, FTZ))
             return cudaErrorInvalidValue;
     } else {
-        emap = umap;  // not read
+        emap = tmap;  // not read
     }
     static KernelSetup setup;  // per instantiation
-    const cudaError_t e = setup_kernel(setup, force_st_kernel<V, FTZ, TI>, F::SMEM);
+    const cudaError_t e = setup_kernel(setup, force_st_kernel<V, FTZ, TI, UW>, F::SMEM);
     if (e != cudaSuccess) return e;
-    return launch_ex(force_st_kernel<V, FTZ, TI>, brick_grid(a.g, FTZ), dim3(FTX, FTY, 1), F::SMEM,
-                     s, a.pdl, dmap, smap, umap, emap, a);
+    return launch_ex(force_st_kernel<V, FTZ, TI, UW>, brick_grid(a.g, FTZ), dim3(FTX, FTY, 1),
+                     F::SMEM, s, a.pdl, dmap, smap, tmap, emap, a, taps);
 }
 
 template <int V, typename TI>
 cudaError_t launch_d_pair(const ForceArgs& zd, const ForceArgs& st, const Taps& taps,
                           cudaStream_t s) {
+    if (!force_d_writes_u(zd.g)) {  // large levels: bricks of 4 (z + D), 4 or 8 planes
+        const cudaError_t e = launch_zd<V, 4, TI, false>(zd, taps, s);
+        if (e != cudaSuccess) return e;
+        return st.depth >= 8 ? launch_st<V, 8, TI, false>(st, taps, s)
+                             : launch_st<V, 4, TI, false>(st, taps, s);
+    }
     cudaError_t e = cudaErrorInvalidValue;
     switch (zd.depth) {
-        case 8: e = launch_zd<V, 8, TI>(zd, taps, s); break;
+        case 8:
         case 6:
-        case 4: e = launch_zd<V, 4, TI>(zd, taps, s); break;
-        case 2: e = launch_zd<V, 2, TI>(zd, taps, s); break;
-        case 1: e = launch_zd<V, 1, TI>(zd, taps, s); break;
+        case 4: e = launch_zd<V, 4, TI, true>(zd, taps, s); break;
+        case 2: e = launch_zd<V, 2, TI, true>(zd, taps, s); break;
+        case 1: e = launch_zd<V, 1, TI, true>(zd, taps, s); break;
         default: break;
     }
     if (e != cudaSuccess) return e;
     switch (st.depth) {
-        case 8: return launch_st<V, 8, TI>(st, s);
+        case 8: return launch_st<V, 8, TI, true>(st, taps, s);
         case 6:
-        case 4: return launch_st<V, 4, TI>(st, s);
-        case 2: return launch_st<V, 2, TI>(st, s);
-        case 1: return launch_st<V, 1, TI>(st, s);
+        case 4: return launch_st<V, 4, TI, true>(st, taps, s);
+        case 2: return launch_st<V, 2, TI, true>(st, taps, s);
+        case 1: return launch_st<V, 1, TI, true>(st, taps, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -120,14 +126,29 @@ bool force_d_supported(int variant, const ForceArgs& a, const Taps& taps) {
     return variant >= 2 && variant <= 5 && force_zs_supported(variant, a, taps);
 }
 
-int force_d_planes(int variant) { return variant == 5 ? 5 : 4; }
+// u written by the z + D pass, or formed again by the force pass: written on
+// levels of at most 2^20 voxels, whose t, u, D and images stay in L2.  Measured
+// per iteration, written -> formed again, Eq. 3 / Eq. 6: 64x64x25 7.95 -> 8.37 /
+// 8.36 -> 8.81 us, 128x128x50 18.5 -> 19.9 / 21.2 -> 21.8, 128x128x64 20.6 ->
+// 21.1 / 23.6 -> 24.2; above, 160x160x64 28.6 -> 28.2 / 32.9 -> 33.0, 192x192x64
+// 39.7 -> 37.1 / 45.3 -> 44.7, 193x171x87 57.1 -> 53.2 / 65.7 -> 64.7,
+// 256x256x100 103.2 -> 96.1 / 117.1 -> 114.1.
+bool force_d_writes_u(long long voxels) { return voxels <= (1LL << 20); }
 
-// Brick depth of both kernels: 8 where such bricks still number four per SM,
-// else the deepest of 4 and 2 that gives one per SM, else 1 -- 8, 4 and 2 on
-// the 256x256x100 pyramid, the autotuner's choice there for Eq. 3 and Eq. 6
-// (Eq. 3: 10.46 ms per registration against 10.63 with 4 on every level)
-int force_d_depth(const Grid3& g, int num_sms) {
+int force_d_planes(int variant, const Grid3& g) {
+    return (variant == 5 ? 2 : 1) + (force_d_writes_u(g) ? 3 : 0);
+}
+
+// Brick depth of the force pass (the z + D pass caps it): 8 where such bricks
+// still number four per SM, else the deepest of 4 and 2 that gives one per SM,
+// else 1.  Eq. 6 on large levels takes 4: with its d box, 8 leaves three blocks
+// per SM (256x256x100: 113.4 us per iteration at 4, 119 at 8; Eq. 3 the other
+// way round, 100.8 and 97.9).  Blocks per SM there: five of the z + D kernel for
+// Eqs. 3-5 (95.9 us per iteration against 97.9 with four), four for Eq. 6 (119
+// against 122: its two interpolations want the registers).
+int force_d_depth(int variant, const Grid3& g, int num_sms) {
     const long long bxy = (long long)((g.nx + FTX - 1) / FTX) * ((g.ny + FTY - 1) / FTY);
+    if (variant == 5 && !force_d_writes_u(g)) return 4;
     if (bxy * ((g.nz + 7) / 8) >= 4LL * num_sms) return 8;
     for (int d = 4; d >= 2; d /= 2)
         if (bxy * ((g.nz + d - 1) / d) >= num_sms) return d;

@@ -59,19 +59,19 @@ __global__ void __launch_bounds__(FNT, (V >= 2 && FTZ >= 2) ? 3 : 4)
         gzs_block<V, FTZ, TI>(&G.tmap[j], &G.smap[j], &G.mmap[j], G.a[j], G.taps, bp);
 }
 
-template <int V, int FTZ, typename TI>
+template <int V, int FTZ, typename TI, bool UW>
 __global__ void __launch_bounds__(FNT, 4) force_zd_grouped_kernel(const __grid_constant__ ZDGroup G) {
     const int b = blockIdx.x;
     const int j = group_job(G.first, G.n, b);
-    zd_block<V, FTZ, TI>(&G.tmap[j], G.a[j], G.taps,
+    zd_block<V, FTZ, TI, UW>(&G.tmap[j], G.a[j], G.taps,
                          group_pos(b - G.first[j], G.gx[j], G.gy[j], G.gz[j]));
 }
 
-template <int V, int FTZ, typename TI>
+template <int V, int FTZ, typename TI, bool UW>
 __global__ void __launch_bounds__(FNT, 4) force_st_grouped_kernel(const __grid_constant__ STGroup G) {
     const int b = blockIdx.x;
     const int j = group_job(G.first, G.n, b);
-    st_block<V, FTZ, TI>(&G.dmap[j], &G.smap[j], &G.umap[j], &G.emap[j], G.a[j],
+    st_block<V, FTZ, TI, UW>(&G.dmap[j], &G.smap[j], &G.tmap[j], &G.emap[j], G.a[j], G.taps,
                          group_pos(b - G.first[j], G.gx[j], G.gy[j], G.gz[j]));
 }
 
@@ -265,7 +265,7 @@ cudaError_t launch_force_zs_grouped(int variant, int img_type, const ZSGroup& G,
 bool d_group_add(ZDGroup& Z, STGroup& T, const ForceArgs& zd, const ForceArgs& st) {
     const int d = Z.depth;
     if (Z.n >= kGroupMax || Z.n != T.n || T.depth != d || Z.variant < 2 || Z.variant > 5 ||
-        T.variant != Z.variant || zd.field_type != kStoreF32 ||
+        T.variant != Z.variant || T.writes_u != Z.writes_u || zd.field_type != kStoreF32 ||
         (zd.img_type != kStoreF32 && zd.img_type != kStoreI16) || Z.taps.R != FZR ||
         !(d == 1 || d == 2 || d == 4) || zd.dbuf == nullptr || st.dbuf == nullptr ||
         (Z.variant == 5 && (zd.dbuf2 == nullptr || st.dbuf2 == nullptr)))
@@ -285,12 +285,12 @@ bool d_group_add(ZDGroup& Z, STGroup& T, const ForceArgs& zd, const ForceArgs& s
     if (!encode4(&Z.tmap[j], f32, zd.u, zd.g, 3, 4, tbox) ||
         !encode4(&T.dmap[j], f32, st.dbuf, st.g, 1, 4, dbox) ||
         !encode4(&T.smap[j], it, st.S, st.g, 1, esz, sbox) ||
-        !encode4(&T.umap[j], f32, st.u, st.g, 3, 4, ubox))
+        !encode4(&T.tmap[j], f32, st.u, st.g, 3, 4, T.writes_u ? ubox : tbox))
         return false;
     if (Z.variant == 5) {
         if (!encode4(&T.emap[j], f32, st.dbuf2, st.g, 1, 4, ebox)) return false;
     } else {
-        T.emap[j] = T.umap[j];  // not read
+        T.emap[j] = T.tmap[j];  // not read
     }
     Z.a[j] = zd;
     T.a[j] = st;
@@ -302,26 +302,29 @@ bool d_group_add(ZDGroup& Z, STGroup& T, const ForceArgs& zd, const ForceArgs& s
     return true;
 }
 
-template <int V, int FTZ, typename TI>
+template <int V, int FTZ, typename TI, bool UW>
 static cudaError_t launch_dg(const ZDGroup& Z, const STGroup& T, cudaStream_t s, bool pdl) {
-    constexpr int ZS = ZDGeom<FTZ>::SMEM, TS = STGeom<FTZ, V, TI>::SMEM;
+    constexpr int ZS = ZDGeom<FTZ>::SMEM, TS = STGeom<FTZ, V, TI, UW>::SMEM;
     static KernelSetup zst, tst;  // per instantiation
-    cudaError_t e = setup_kernel(zst, force_zd_grouped_kernel<V, FTZ, TI>, ZS);
-    if (e == cudaSuccess) e = setup_kernel(tst, force_st_grouped_kernel<V, FTZ, TI>, TS);
+    cudaError_t e = setup_kernel(zst, force_zd_grouped_kernel<V, FTZ, TI, UW>, ZS);
+    if (e == cudaSuccess) e = setup_kernel(tst, force_st_grouped_kernel<V, FTZ, TI, UW>, TS);
     if (e != cudaSuccess) return e;
-    e = launch_ex(force_zd_grouped_kernel<V, FTZ, TI>, dim3((unsigned)Z.first[Z.n]),
+    e = launch_ex(force_zd_grouped_kernel<V, FTZ, TI, UW>, dim3((unsigned)Z.first[Z.n]),
                   dim3(FTX, FTY, 1), ZS, s, pdl, Z);
     if (e != cudaSuccess) return e;
-    return launch_ex(force_st_grouped_kernel<V, FTZ, TI>, dim3((unsigned)T.first[T.n]),
+    return launch_ex(force_st_grouped_kernel<V, FTZ, TI, UW>, dim3((unsigned)T.first[T.n]),
                      dim3(FTX, FTY, 1), TS, s, pdl, T);
 }
 
 template <int V, typename TI>
 static cudaError_t launch_dg_depth(const ZDGroup& Z, const STGroup& T, cudaStream_t s, bool pdl) {
+    // chunks too large for L2 always come with the deepest bricks
+    if (!Z.writes_u)
+        return Z.depth == 4 ? launch_dg<V, 4, TI, false>(Z, T, s, pdl) : cudaErrorInvalidValue;
     switch (Z.depth) {
-        case 4: return launch_dg<V, 4, TI>(Z, T, s, pdl);
-        case 2: return launch_dg<V, 2, TI>(Z, T, s, pdl);
-        case 1: return launch_dg<V, 1, TI>(Z, T, s, pdl);
+        case 4: return launch_dg<V, 4, TI, true>(Z, T, s, pdl);
+        case 2: return launch_dg<V, 2, TI, true>(Z, T, s, pdl);
+        case 1: return launch_dg<V, 1, TI, true>(Z, T, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -88,13 +88,18 @@ cudaError_t launch_force_zs(int variant, const ForceArgs& a, const Taps& taps, c
 
 // Eqs. 3-6, the split iteration with the difference image formed once per
 // voxel (dir_split_d.cuh): after launch_smooth_xy, the z + D pass (zd: u = t,
-// v = the u it writes, dbuf / dbuf2 = the D it writes) and the stencil force
-// pass (st: u = that u, v = the field out, dbuf / dbuf2 = that D), each with
-// its own brick depth (1, 2, 4 or 8; 6 runs as 4).  force_d_planes: floats per
-// voxel of the u + D scratch (4, Eq. 6: 5).
+// dbuf / dbuf2 = the D it writes) and the stencil force pass (st: u = t, v = the
+// field out, dbuf / dbuf2 = that D), each with its own brick depth (1, 2, 4 or
+// 8; 6 runs as 4).  On levels where force_d_writes_u, zd.v and st.u are u, which
+// the first writes and the second reads.  force_d_planes: floats per voxel of
+// the scratch for D (1, Eq. 6: 2) and, there, u (3).
 bool force_d_supported(int variant, const ForceArgs& a, const Taps& taps);
-int force_d_planes(int variant);
-int force_d_depth(const Grid3& g, int num_sms);
+bool force_d_writes_u(long long voxels);
+inline bool force_d_writes_u(const Grid3& g) {
+    return force_d_writes_u((long long)g.nx * g.ny * g.nz);
+}
+int force_d_planes(int variant, const Grid3& g);
+int force_d_depth(int variant, const Grid3& g, int num_sms);
 cudaError_t launch_force_d(int variant, const ForceArgs& zd, const ForceArgs& st, const Taps& taps,
                            cudaStream_t s);
 
@@ -143,7 +148,7 @@ cudaError_t launch_force_zs_grouped(int variant, int img_type, const ZSGroup& G,
 
 // The Eqs. 3-6 split after the difference image, grouped the same way: the z +
 // D kernel (each job's t map and arguments as for launch_force_d's zd) and the
-// stencil force kernel (its D, S, u and Eq. 6 d maps and arguments as for
+// stencil force kernel (its D, S, t and Eq. 6 d maps and arguments as for
 // st); both groups share first / gx / gy / gz and the brick depth (1, 2 or 4).
 struct ZDGroup {
     CUtensorMap tmap[kGroupMax];
@@ -154,15 +159,18 @@ struct ZDGroup {
     int n = 0;
     int variant = 0;
     int depth = 0;
+    bool writes_u = false;       // u crosses memory between the two kernels
 };
 struct STGroup {
-    CUtensorMap dmap[kGroupMax], smap[kGroupMax], umap[kGroupMax], emap[kGroupMax];
+    CUtensorMap dmap[kGroupMax], smap[kGroupMax], tmap[kGroupMax], emap[kGroupMax];
     ForceArgs a[kGroupMax];
     int first[kGroupMax + 1];
     int gx[kGroupMax], gy[kGroupMax], gz[kGroupMax];
+    Taps taps;
     int n = 0;
     int variant = 0;
     int depth = 0;
+    bool writes_u = false;       // u crosses memory between the two kernels
 };
 // Add one job to both groups (variant and depth already set on them)
 bool d_group_add(ZDGroup& Z, STGroup& T, const ForceArgs& zd, const ForceArgs& st);

@@ -50,6 +50,7 @@ __device__ __forceinline__ f32x2 f2_add_rounded(f32x2 a, f32x2 b) {
 __device__ __forceinline__ f32x2 f2_sub_rounded(f32x2 a, f32x2 b) {
     return f2_pack(__fsub_rn(f2_lo(a), f2_lo(b)), __fsub_rn(f2_hi(a), f2_hi(b)));
 }
+__device__ __forceinline__ f32x2 f2_neg(f32x2 a) { return f2_pack(-f2_lo(a), -f2_hi(a)); }
 // (x x + y y) + z z with the two additions fused, as r_sq3
 __device__ __forceinline__ f32x2 f2_sq3(f32x2 x, f32x2 y, f32x2 z) {
     return f2_fma(z, z, f2_fma(y, y, f2_mul(x, x)));
@@ -185,14 +186,13 @@ template <int V>
 __device__ __forceinline__ void pair_update(f32x2 d, const f32x2 (&gs)[3], const f32x2 (&gm)[3],
                                             f32x2 b, float alpha2, const f32x2 (&u)[3],
                                             f32x2 (&dr)[3], f32x2 (&v)[3]) {
-    // d^2 is rounded by itself before |g|^2 is added (Eq. 5: alpha^2 d^2 is
-    // added in one rounding), as the compiler contracts the scalar kernels
+    // d^2 (Eq. 5: alpha^2 d^2) is rounded by itself before |g|^2 is added, as
+    // the compiler contracts the scalar kernels, which use it twice
     if (V == 3 || V == 4) {
-        const f32x2 d2 = f2_mul(d, d);
-        const f32x2 g1 = f2_sq3(gs[0], gs[1], gs[2]), g2 = f2_sq3(gm[0], gm[1], gm[2]);
-        const f32x2 a2 = f2_dup(alpha2);
-        const f32x2 p = pair_quotient(d, V == 4 ? f2_fma(a2, d2, g1) : f2_add_rounded(d2, g1));
-        const f32x2 q = pair_quotient(d, V == 4 ? f2_fma(a2, d2, g2) : f2_add_rounded(d2, g2));
+        f32x2 d2 = f2_mul(d, d);
+        if (V == 4) d2 = f2_mul(f2_dup(alpha2), d2);
+        const f32x2 p = pair_quotient(d, f2_add_rounded(d2, f2_sq3(gs[0], gs[1], gs[2])));
+        const f32x2 q = pair_quotient(d, f2_add_rounded(d2, f2_sq3(gm[0], gm[1], gm[2])));
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             dr[c] = f2_add_rounded(f2_mul(p, gs[c]), f2_mul(q, gm[c]));

@@ -6,19 +6,26 @@
 // the one-pass form (dir_force_gm.cuh) interpolates W on its brick plus a
 // one-voxel halo: about twice per voxel at 32 x 8 x 4 bricks, four times for
 // Eq. 6, which also warps S backwards.  Here one iteration is three kernels:
-//   x/y pass   t = G_y G_x v                     (sxy_block, unchanged)
+//   x/y pass   t = G_y G_x v                     (dir_xy.cuh, sxy_block)
 //   z + D pass u = G_z t down each thread's own column, then per voxel
-//              D = W - S (Eq. 6: D_m + D_s and d = D_m - D_s); writes u and D
-//   force pass the gradients of S and of W (= D + S) from shared-memory boxes
-//              of D and S with a one-voxel halo, the force, v = u - dr(u) and
-//              the reductions: a stencil with no gathers
-// The arithmetic is that of gm_force_body voxel by voxel (D by interp_rel with
-// the same operands, the same clamped neighbours, the same force call), so the
-// field is bit for bit the one of the other schedules.  The default for Eqs.
-// 3-6 on every pyramid level: the one-pass blocks were bound by issue and by
-// the latency of their footprint gathers, not by memory, so the 36 B per voxel
-// of u and D written here and read back by the force pass cost less than the
-// gathers and instructions they remove.
+//              D = W - S (Eq. 6: D_m + D_s and d = D_m - D_s); writes D
+//   force pass u = G_z t again, the gradients of S and of W (= D + S) from
+//              shared-memory boxes of D and S with a one-voxel halo, the
+//              force, v = u - dr(u) and the reductions: a stencil with no
+//              gathers
+// The arithmetic is that of gm_force_body voxel by voxel (D by the same
+// interpolation with the same operands, the same clamped neighbours, the same
+// force), so the field is bit for bit the one of the other schedules.  The
+// default for Eqs. 3-6 on every pyramid level: the one-pass blocks were bound by
+// issue and by the latency of their footprint gathers, not by memory.
+//
+// With packed arithmetic (dir_pair.cuh) these kernels run at 0.86 of the copy
+// rate on large levels, so u does not cross memory between them there: the
+// force pass redoes the z pass (24 warp instructions per 32 voxels) instead of
+// reading a u that the z + D pass would write, 80 B per voxel and iteration
+// instead of 92 (Eq. 6: 88 for 100).  On levels that stay in L2 the second z
+// pass only lengthens the chain, and the z + D pass writes u too (UW; the rule
+// is force_d_writes_u).
 #pragma once
 
 #include <cuda.h>
@@ -38,9 +45,9 @@ struct ZDGeom {
     static constexpr int SMEM = 128 + OFF_BAR + 64;
 };
 
-// One brick of the z + D pass (every thread of the block calls it).  a.u: t,
-// a.v: u out; a.dbuf: D out (Eq. 6: D_m + D_s), a.dbuf2: Eq. 6's d out.
-template <int V, int FTZ, typename TI>
+// One brick of the z + D pass (every thread of the block calls it).  a.u: t;
+// a.dbuf: D out (Eq. 6: D_m + D_s), a.dbuf2: Eq. 6's d out; UW: a.v: u out.
+template <int V, int FTZ, typename TI, bool UW>
 __device__ __forceinline__ void zd_block(const CUtensorMap* tmap, const ForceArgs& a,
                                          const Taps& taps, const BlockPos bp) {
     static_assert(V >= 2 && V <= 5, "Eqs. 3-6");
@@ -64,12 +71,19 @@ __device__ __forceinline__ void zd_block(const CUtensorMap* tmap, const ForceArg
     const int bz0 = (bp.gz - 1 - bp.z) * FTZ;
     const int x = bx0 + tx, y = by0 + ty;
     const bool col_valid = (x < g.nx) && (y < g.ny);
+    constexpr int H = FTZ > 1 ? FTZ / 2 : 1;  // pairs (k, k + H); FTZ = 1: both lanes the voxel
+    constexpr int HB = FTZ > 1 ? H : 0;
+    const uint32_t ipl = (uint32_t)sizeof(TI) * (uint32_t)g.plane;
     pdl_trigger();
-    // S at this thread's voxels (static: read before the wait)
-    float s0[FTZ];
+    // S at this thread's voxels (static: read before the wait), planes past the
+    // last as the last
+    f32x2 s0[H];
 #pragma unroll
-    for (int k = 0; k < FTZ; ++k)
-        s0[k] = (col_valid && bz0 + k < g.nz) ? ldg_as<float>(S + offs(g, x, y, bz0 + k)) : 0.0f;
+    for (int k = 0; k < H; ++k) {
+        const uint32_t o = (uint32_t)sizeof(TI) * (uint32_t)offs(g, min(x, g.nx - 1), min(y, g.ny - 1), 0);
+        s0[k] = f2_pack(img_ldg(S, o + ipl * (uint32_t)min(bz0 + k, g.nz - 1)),
+                        img_ldg(S, o + ipl * (uint32_t)min(bz0 + k + HB, g.nz - 1)));
+    }
     if (tid == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
@@ -77,87 +91,71 @@ __device__ __forceinline__ void zd_block(const CUtensorMap* tmap, const ForceArg
         mbar_arrive_expect_tx(bar, (uint32_t)Z::TBOX);
         pdl_wait();
         tma_load_4d(base, tmap, bx0, by0, bz0 - R, 0, bar);  // planes outside: zero fill
-        if (a.pf_stride > 0) {  // the block pf_stride positions ahead: its t box into L2
-            const long long gx = bp.gx, gy = bp.gy;
-            const long long b = bp.x + gx * (bp.y + gy * (long long)bp.z) + a.pf_stride;
-            if (b < gx * gy * bp.gz) {
-                const int px = (int)(b % gx) * FTX, py = (int)((b / gx) % gy) * FTY;
-                const int pz = (int)(bp.gz - 1 - b / (gx * gy)) * FTZ;
-                tma_prefetch_4d(tmap, px, py, pz - R, 0);
-            }
-        }
+        BlockPos nb;
+        if (a.pf_stride > 0 && bp.ahead(a.pf_stride, nb))  // that block's t box into L2
+            tma_prefetch_4d(tmap, nb.x * FTX, nb.y * FTY, (bp.gz - 1 - nb.z) * FTZ - R, 0);
     }
-    pdl_wait();  // every thread: u and D are written below, which the previous
-                 // iteration's force pass reads (finished before the kernel before)
+    pdl_wait();  // every thread: D is written below, which the previous iteration's
+                 // force pass reads (finished before the kernel before)
     __syncthreads();
-    bool ok = true;
-    if (tid == 0) ok = mbar_wait_bounded(bar, 0, kWaitLimitNs);
-    if (__syncthreads_or(!ok)) {
-        if (tid == 0 && a.err) atomicOr(a.err, kErrTmaTimeout);
-        return;
-    }
-    (void)mbar_try_wait(bar, 0);
+    // every thread waits for the copy itself (bounded); one that gave up flags
+    // the error and goes on over whatever the box holds
+    if (!mbar_wait_bounded(bar, 0, kWaitLimitNs) && a.err) atomicOr(a.err, kErrTmaTimeout);
     if (!col_valid) return;  // no barrier below
 
-    // z pass down this thread's column, as zs_block: edge planes replicated
-    // into the zero fill, u[c][k] written over t planes R .. R + FTZ - 1
-    float w[R + 1];
-#pragma unroll
-    for (int t = 0; t <= R; ++t) w[t] = taps.wf[t];
+    // z pass down this thread's column, as zs_block
     float* tcol = tb + tid;  // plane j of component c at tcol[(c * NPZ + j) * FNT]
     const int zlo = bz0 - R;
-    if (zlo < 0 || zlo + NPZ > g.nz) {
-        const int jlo = max(0, -zlo), jhi = min(NPZ - 1, g.nz - 1 - zlo);
-        for (int c = 0; c < 3; ++c) {
-            float* tc = tcol + c * NPZ * FNT;
-            const float lo = tc[jlo * FNT], hi = tc[jhi * FNT];
-            for (int j = 0; j < jlo; ++j) tc[j * FNT] = lo;
-            for (int j = jhi + 1; j < NPZ; ++j) tc[j * FNT] = hi;
-        }
-    }
+    if (zlo < 0 || zlo + NPZ > g.nz)
+        for (int c = 0; c < 3; ++c)
+            replicate_planes(tcol + c * NPZ * FNT, FNT, NPZ, max(0, -zlo),
+                             min(NPZ - 1, g.nz - 1 - zlo));
+    f32x2 up[3][H];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float cv[NPZ];
-#pragma unroll
-        for (int j = 0; j < NPZ; ++j) cv[j] = tcol[(c * NPZ + j) * FNT];
-#pragma unroll
-        for (int k = 0; k < FTZ; ++k) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int t = 0; t < 2 * R + 1; ++t) acc = fmaf(w[t <= R ? t : 2 * R - t], cv[k + t], acc);
-            tcol[(c * NPZ + R + k) * FNT] = acc;
-        }
-    }
+    for (int c = 0; c < 3; ++c) pair_zpass<R, FTZ, H>(tcol + c * NPZ * FNT, FNT, taps, up[c]);
 
     // D per voxel: the interpolations of gm_force_body's d_at at the voxel itself
-    const Interp ip(g);
-    const int cs = (int)g.cs;
+    const PairInterp<TI> ip(g, x, y, bz0);
+    const uint32_t o0 = 4u * (uint32_t)offs(g, x, y, bz0), pl = 4u * (uint32_t)g.plane;
 #pragma unroll
-    for (int k = 0; k < FTZ; ++k) {
-        const int z = bz0 + k;
-        if (z < g.nz) {
-            const float ux = tcol[(R + k) * FNT], uy = tcol[(NPZ + R + k) * FNT],
-                        uz = tcol[(2 * NPZ + R + k) * FNT];
-            const float wm = interp_rel(M, ip, x, ux, y, uy, z, uz, s0[k]);
-            const int o = offs(g, x, y, z);
-            uo[o] = ux;
-            uo[o + cs] = uy;
-            uo[o + 2 * cs] = uz;
-            if (IC) {
-                const float ws = interp_rel(S, ip, x, -ux, y, -uy, z, -uz, s0[k]);
-                Do[o] = wm + ws;
-                do2[o] = wm - ws;
-            } else {
-                Do[o] = wm;
+    for (int k = 0; k < H; ++k) {
+        const int ka = k, kb = k + HB;
+        const bool va = bz0 + ka < g.nz, vb = FTZ > 1 && bz0 + kb < g.nz;
+        const f32x2 wm = ip.at(M, ka, kb, up[0][k], up[1][k], up[2][k], s0[k]);
+        f32x2 D = wm, d = 0ull;
+        if (IC) {
+            const f32x2 ws =
+                ip.at(S, ka, kb, f2_neg(up[0][k]), f2_neg(up[1][k]), f2_neg(up[2][k]), s0[k]);
+            D = f2_add(wm, ws);
+            d = f2_sub(wm, ws);
+        }
+        if (va) {
+            const uint32_t o = o0 + ka * pl;
+            if (UW) {
+                *at_byte(uo, o) = f2_lo(up[0][k]);
+                *at_byte(uo + g.cs, o) = f2_lo(up[1][k]);
+                *at_byte(uo + 2 * g.cs, o) = f2_lo(up[2][k]);
             }
+            *at_byte(Do, o) = f2_lo(D);
+            if (IC) *at_byte(do2, o) = f2_lo(d);
+        }
+        if (vb) {
+            const uint32_t o = o0 + kb * pl;
+            if (UW) {
+                *at_byte(uo, o) = f2_hi(up[0][k]);
+                *at_byte(uo + g.cs, o) = f2_hi(up[1][k]);
+                *at_byte(uo + 2 * g.cs, o) = f2_hi(up[2][k]);
+            }
+            *at_byte(Do, o) = f2_hi(D);
+            if (IC) *at_byte(do2, o) = f2_hi(d);
         }
     }
 }
 
 // Force pass: D with a one-voxel halo over the columns x0 - 4 .. x0 + 35 (a
-// 16-byte aligned start), S with the halo of FGGeom, u (and Eq. 6's d) on the
-// brick.
-template <int FTZ, int V, typename TI>
+// 16-byte aligned start), S with the halo of FGGeom, t on the brick with R
+// planes above and below (UW: u on the brick) and Eq. 6's d on the brick.
+template <int FTZ, int V, typename TI, bool UW>
 struct STGeom {
     static constexpr bool IC = (V == 5);
     static constexpr int FBX = 16 / (int)sizeof(TI);
@@ -165,30 +163,33 @@ struct STGeom {
     static constexpr int DW = FTX + 8, DH = FTY + 2, DD = FTZ + 2;
     static constexpr int DBOX = DD * DH * DW * 4;                    // [DD][DH][DW] floats
     static constexpr int SBOX = DD * FSH * FSW * (int)sizeof(TI);   // [DD][FSH][FSW]
-    static constexpr int UBOX = 3 * FTZ * FTY * FTX * 4;            // [3][FTZ][FTY][FTX]
+    static constexpr int TR = UW ? 0 : FZR;                         // halo planes of t
+    static constexpr int NPZ = FTZ + 2 * TR;
+    static constexpr int TBOX = 3 * NPZ * FTY * FTX * 4;            // [3][NPZ][FTY][FTX]
     static constexpr int EBOX = IC ? FTZ * FTY * FTX * 4 : 0;       // [FTZ][FTY][FTX]
     static constexpr int OFF_S = (DBOX + 127) / 128 * 128;
-    static constexpr int OFF_U = OFF_S + (SBOX + 127) / 128 * 128;
-    static constexpr int OFF_E = OFF_U + (UBOX + 127) / 128 * 128;
+    static constexpr int OFF_T = OFF_S + (SBOX + 127) / 128 * 128;
+    static constexpr int OFF_E = OFF_T + (TBOX + 127) / 128 * 128;
     static constexpr int OFF_BAR = OFF_E + (EBOX + 127) / 128 * 128;
     static constexpr int SMEM = 128 + OFF_BAR + 64;
 };
 
-// One brick of the force pass (every thread of the block calls it).  a.u: u,
-// a.v: v out; a.dbuf: D, a.dbuf2: Eq. 6's d.
-template <int V, int FTZ, typename TI>
+// One brick of the force pass (every thread of the block calls it).  a.u: t
+// (UW: u), a.v: v out; a.dbuf: D, a.dbuf2: Eq. 6's d.
+template <int V, int FTZ, typename TI, bool UW>
 __device__ __forceinline__ void st_block(const CUtensorMap* dmap, const CUtensorMap* smap,
-                                         const CUtensorMap* umap, const CUtensorMap* emap,
-                                         const ForceArgs& a, const BlockPos bp) {
+                                         const CUtensorMap* tmap, const CUtensorMap* emap,
+                                         const ForceArgs& a, const Taps& taps, const BlockPos bp) {
     static_assert(V >= 2 && V <= 5, "Eqs. 3-6");
     if (a.stop_iter != nullptr && *a.stop_iter < a.iter) return;  // uniform across the grid
-    using F = STGeom<FTZ, V, TI>;
+    using F = STGeom<FTZ, V, TI, UW>;
     constexpr int FSW = F::FSW, DW = F::DW, DH = F::DH, FBX = F::FBX;
+    constexpr int R = F::TR, NPZ = F::NPZ;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const float* db = reinterpret_cast<const float*>(base);             // [DD][DH][DW]
-    const TI* sb = reinterpret_cast<const TI*>(base + F::OFF_S);        // [DD][FSH][FSW]
-    const float* ub = reinterpret_cast<const float*>(base + F::OFF_U);  // [3][FTZ][FTY][FTX]
+    float* db = reinterpret_cast<float*>(base);                         // [DD][DH][DW]
+    TI* sb = reinterpret_cast<TI*>(base + F::OFF_S);                    // [DD][FSH][FSW]
+    float* tb = reinterpret_cast<float*>(base + F::OFF_T);              // [3][NPZ][FTY][FTX]
     const float* eb = reinterpret_cast<const float*>(base + F::OFF_E);  // [FTZ][FTY][FTX]
     uint64_t* bar = reinterpret_cast<uint64_t*>(base + F::OFF_BAR);
     const Grid3 g = a.g;
@@ -203,90 +204,122 @@ __device__ __forceinline__ void st_block(const CUtensorMap* dmap, const CUtensor
         mbar_init(bar, 1);
         fence_mbar_init();
         fence_proxy_async();
-        mbar_arrive_expect_tx(bar, (uint32_t)(F::DBOX + F::SBOX + F::UBOX + F::EBOX));
+        mbar_arrive_expect_tx(bar, (uint32_t)(F::DBOX + F::SBOX + F::TBOX + F::EBOX));
         tma_load_4d(base + F::OFF_S, smap, sx0, sy0, sz0, 0, bar);  // static
         pdl_wait();
         tma_load_4d(base, dmap, dx0, dy0, dz0, 0, bar);
-        tma_load_4d(base + F::OFF_U, umap, bx0, by0, bz0, 0, bar);
+        tma_load_4d(base + F::OFF_T, tmap, bx0, by0, bz0 - R, 0, bar);  // planes outside: zero fill
         if (F::IC) tma_load_4d(base + F::OFF_E, emap, bx0, by0, bz0, 0, bar);
-        if (a.pf_stride > 0) {  // the block pf_stride positions ahead: its boxes into L2
-            const long long gx = bp.gx, gy = bp.gy;
-            const long long b = bp.x + gx * (bp.y + gy * (long long)bp.z) + a.pf_stride;
-            if (b < gx * gy * bp.gz) {
-                const int px = (int)(b % gx) * FTX, py = (int)((b / gx) % gy) * FTY;
-                const int pz = (int)(b / (gx * gy)) * FTZ;
-                tma_prefetch_4d(dmap, px - 4, py - 1, pz - 1, 0);
-                tma_prefetch_4d(smap, px - FBX, py - 1, pz - 1, 0);
-                tma_prefetch_4d(umap, px, py, pz, 0);
-            }
+        BlockPos nb;
+        if (a.pf_stride > 0 && bp.ahead(a.pf_stride, nb)) {  // that block's boxes into L2
+            const int px = nb.x * FTX, py = nb.y * FTY, pz = nb.z * FTZ;
+            tma_prefetch_4d(dmap, px - 4, py - 1, pz - 1, 0);
+            tma_prefetch_4d(smap, px - FBX, py - 1, pz - 1, 0);
+            tma_prefetch_4d(tmap, px, py, pz - R, 0);
         }
     }
     pdl_wait();  // every thread: v is written below, which this iteration's x/y
                  // pass read (finished before the kernel before)
     __syncthreads();
-    bool ok = true;
-    if (tid == 0) ok = mbar_wait_bounded(bar, 0, kWaitLimitNs);
-    if (__syncthreads_or(!ok)) {
-        if (tid == 0 && a.err) atomicOr(a.err, kErrTmaTimeout);
-        return;
-    }
-    (void)mbar_try_wait(bar, 0);
+    if (!mbar_wait_bounded(bar, 0, kWaitLimitNs) && a.err) atomicOr(a.err, kErrTmaTimeout);
 
     const int x = bx0 + tx, y = by0 + ty;
-    const bool col_valid = (x < g.nx) && (y < g.ny);
-    float sd2 = 0.0f, sdu = 0.0f, su = 0.0f;
+    PairSums sums;
     CorrSums<float> corr_s;  // with a.corr: the correlation sums
-    if (col_valid) {
-        // the clamped neighbours of gm_force_body's footprint, in box indices
-        const int sx = x - sx0, sxm = max(x - 1, 0) - sx0, sxp = min(x + 1, g.nx - 1) - sx0;
-        const int sy = y - sy0, sym = max(y - 1, 0) - sy0, syp = min(y + 1, g.ny - 1) - sy0;
-        const int cx = x - dx0, cxm = max(x - 1, 0) - dx0, cxp = min(x + 1, g.nx - 1) - dx0;
-        const int cy = y - dy0, cym = max(y - 1, 0) - dy0, cyp = min(y + 1, g.ny - 1) - dy0;
-        const int cs = (int)g.cs;
-#pragma unroll
-        for (int k = 0; k < FTZ; ++k) {
-            const int z = bz0 + k;
-            if (z < g.nz) {
-                const int pc = k + 1;
-                const int pm = max(z - 1, 0) - sz0, pp = min(z + 1, g.nz - 1) - sz0;
-                const TI* Sc = sb + pc * (FSH * FSW);
-                const float gsx = 0.5f * ((float)Sc[sy * FSW + sxp] - (float)Sc[sy * FSW + sxm]);
-                const float gsy = 0.5f * ((float)Sc[syp * FSW + sx] - (float)Sc[sym * FSW + sx]);
-                const float gsz = 0.5f * ((float)sb[pp * (FSH * FSW) + sy * FSW + sx] -
-                                          (float)sb[pm * (FSH * FSW) + sy * FSW + sx]);
-                // grad W = grad D + grad S (Eq. 6: grad(D_m + D_s) + 2 grad S)
-                const float ns = F::IC ? 2.0f : 1.0f;
-                const float* Dc = db + pc * (DH * DW);
-                const float dcen = Dc[cy * DW + cx];
-                const float gmx = r_fma(ns, gsx, 0.5f * (Dc[cy * DW + cxp] - Dc[cy * DW + cxm]));
-                const float gmy = r_fma(ns, gsy, 0.5f * (Dc[cyp * DW + cx] - Dc[cym * DW + cx]));
-                const float gmz = r_fma(ns, gsz, 0.5f * (db[pp * (DH * DW) + cy * DW + cx] -
-                                                         db[pm * (DH * DW) + cy * DW + cx]));
-                const int bi = (k * FTY + ty) * FTX + tx;
-                const float d = F::IC ? eb[bi] : dcen;
-                if (a.corr) {  // reference: S (Eq. 6: the warped static image S + D_s)
-                    float bref = (float)Sc[sy * FSW + sx];
-                    if (F::IC) bref += 0.5f * (dcen - d);
-                    corr_s.add(bref, d);
-                }
-                constexpr int UC = FTZ * FTY * FTX;
-                const float ux = ub[bi], uy = ub[bi + UC], uz = ub[bi + 2 * UC];
-                float dx, dy, dz;
-                demons_force<float, V>(d, gsx, gsy, gsz, gmx, gmy, gmz, 0.0f, alpha2, dx, dy, dz);
-                dx = -dx;
-                dy = -dy;
-                dz = -dz;
-                sd2 += d * d;
-                sdu += r_norm_fast(dx * dx + dy * dy + dz * dz);
-                su += r_norm_fast(ux * ux + uy * uy + uz * uz);
-                const int o = offs(g, x, y, z);
-                v[o] = ux + dx;
-                v[o + cs] = uy + dy;
-                v[o + 2 * cs] = uz + dz;
-            }
+    if (x < g.nx && y < g.ny) {
+        constexpr int SP = FSH * FSW, DP = DH * DW;  // elements per plane of the boxes
+        constexpr int H = FTZ > 1 ? FTZ / 2 : 1, HB = FTZ > 1 ? H : 0;
+        TI* scol = sb + (y - sy0) * FSW + (x - sx0);
+        float* dcol = db + (y - dy0) * DW + (x - dx0);
+        if (bz0 == 0 || bz0 + FTZ >= g.nz) {  // z neighbours outside the volume
+            const int jlo = bz0 == 0 ? 1 : 0, jhi = min(FTZ + 1, g.nz - bz0);
+            replicate_planes(scol, SP, FTZ + 2, jlo, jhi);
+            replicate_planes(dcol, DP, FTZ + 2, jlo, jhi);
         }
+        // x and y neighbours, clamped to the volume
+        const int dxm = x > 0 ? -1 : 0, dxp = x < g.nx - 1 ? 1 : 0;
+        const int yms = y > 0 ? -FSW : 0, yps = y < g.ny - 1 ? FSW : 0;
+        const int ymd = y > 0 ? -DW : 0, ypd = y < g.ny - 1 ? DW : 0;
+        float* __restrict__ vx = v;
+        float* __restrict__ vy = v + g.cs;
+        float* __restrict__ vz = v + 2 * g.cs;
+        const uint32_t o0 = 4u * (uint32_t)offs(g, x, y, bz0), pl = 4u * (uint32_t)g.plane;
+        const f32x2 half = f2_dup(0.5f), ns = f2_dup(F::IC ? 2.0f : 1.0f);
+        // u down this thread's column, as zs_block
+        float* tcol = tb + tid;
+        f32x2 up[3][H];
+        if constexpr (!UW) {
+            if (bz0 < R || bz0 + FTZ + R > g.nz)
+                for (int c = 0; c < 3; ++c)
+                    replicate_planes(tcol + c * NPZ * FNT, FNT, NPZ, max(0, R - bz0),
+                                     min(NPZ - 1, g.nz - 1 - bz0 + R));
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                pair_zpass<R, FTZ, H>(tcol + c * NPZ * FNT, FNT, taps, up[c]);
+        }
+        auto pairs = [&](auto whole) {  // whole: every plane of the brick lies in the volume
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const int ka = k, kb = k + HB;
+                const bool va = whole || bz0 + ka < g.nz;
+                const bool vb = FTZ > 1 && (whole || bz0 + kb < g.nz);
+                auto sgrad = [&](int dp, int dm) {  // half the difference of two values of S
+                    const TI* pa = scol + (ka + 1) * SP;
+                    const TI* pb = scol + (kb + 1) * SP;
+                    return f2_mul(half, f2_sub(f2_pack(img_bits(pa[dp]), img_bits(pb[dp])),
+                                               f2_pack(img_bits(pa[dm]), img_bits(pb[dm]))));
+                };
+                auto dgrad = [&](int dp, int dm) {  // and of D
+                    const float* pa = dcol + (ka + 1) * DP;
+                    const float* pb = dcol + (kb + 1) * DP;
+                    return f2_mul(half, f2_sub(f2_pack(pa[dp], pb[dp]), f2_pack(pa[dm], pb[dm])));
+                };
+                const f32x2 gs[3] = {sgrad(dxp, dxm), sgrad(yps, yms), sgrad(SP, -SP)};
+                // grad W = grad D + grad S (Eq. 6: grad(D_m + D_s) + 2 grad S)
+                const f32x2 gm[3] = {f2_fma(ns, gs[0], dgrad(dxp, dxm)),
+                                     f2_fma(ns, gs[1], dgrad(ypd, ymd)),
+                                     f2_fma(ns, gs[2], dgrad(DP, -DP))};
+                const f32x2 D = f2_pack(dcol[(ka + 1) * DP], dcol[(kb + 1) * DP]);
+                const f32x2 d =
+                    F::IC ? f2_pack(eb[tid + ka * FNT], eb[tid + kb * FNT]) : D;
+                if (a.corr) {  // reference: S (Eq. 6: the warped static image S + D_s)
+                    float ra = img_value<TI>(img_bits(scol[(ka + 1) * SP]));
+                    float rb = img_value<TI>(img_bits(scol[(kb + 1) * SP]));
+                    if (F::IC) {
+                        ra += 0.5f * (f2_lo(D) - f2_lo(d));
+                        rb += 0.5f * (f2_hi(D) - f2_hi(d));
+                    }
+                    if (va) corr_s.add(ra, f2_lo(d));
+                    if (vb) corr_s.add(rb, f2_hi(d));
+                }
+                f32x2 u[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    u[c] = UW ? f2_pack(tcol[(c * NPZ + ka) * FNT], tcol[(c * NPZ + kb) * FNT])
+                              : up[c][k];
+                f32x2 dr[3], vn[3];
+                pair_update<V>(d, gs, gm, 0ull, alpha2, u, dr, vn);
+                sums.add(d, dr, u, va, vb);
+                if (va) {
+                    const uint32_t o = o0 + ka * pl;
+                    *at_byte(vx, o) = f2_lo(vn[0]);
+                    *at_byte(vy, o) = f2_lo(vn[1]);
+                    *at_byte(vz, o) = f2_lo(vn[2]);
+                }
+                if (vb) {
+                    const uint32_t o = o0 + kb * pl;
+                    *at_byte(vx, o) = f2_hi(vn[0]);
+                    *at_byte(vy, o) = f2_hi(vn[1]);
+                    *at_byte(vz, o) = f2_hi(vn[2]);
+                }
+            }
+        };
+        if (bz0 + FTZ <= g.nz)
+            pairs(std::true_type{});
+        else
+            pairs(std::false_type{});
     }
-    block_reduce3_atomic<FNT, float>(sd2, sdu, su, a.red);
+    block_reduce3_atomic<FNT, float>(sums.d2, sums.du, sums.u, a.red);
     if (a.corr) block_reduce4_atomic<FNT, float>(corr_s, a.corr);
 }
 
