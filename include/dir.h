@@ -118,7 +118,10 @@ typedef struct {
                                     differences) to a scratch of 1 (Eq. 6: 2) floats per voxel
                                     of the level, and a stencil kernel forms the force from
                                     them, instead of interpolating W on every brick's halo.
-                                    2 (default): as 4 where it applies.  dir_register_noalloc
+                                    2 (default): as 4 where it applies, and on levels of at most
+                                    16,384 voxels without a stop test or timing all iterations
+                                    in one launch, the field in the shared memory of a
+                                    thread-block cluster.  dir_register_noalloc
                                     has no scratch for the form of 4: there 2 is split for Eqs.
                                     (1)-(2) on every level and for Eqs. (3)-(6) on levels of at
                                     most 2^21 voxels, else fused on the small levels that one
@@ -162,7 +165,8 @@ typedef struct {
     int n_fused_finest;             /* number of launches behind ms_fused_finest */
     int schedule_finest;            /* iteration schedule of level 0: 0 force + smoothing kernels,
                                        1 fused iteration, 2 split Gaussian (fuse = 3), 3 split
-                                       with the difference image (fuse = 4); with a split
+                                       with the difference image (fuse = 4), 4 the whole level
+                                       in one launch (small levels); with a split
                                        schedule ms_smooth_finest times the x/y kernel and
                                        ms_force_finest the z + force kernel (3: the z + D and
                                        the stencil force kernels together) */

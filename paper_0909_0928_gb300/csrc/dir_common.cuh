@@ -192,9 +192,12 @@ __device__ __forceinline__ void block_reduce3_atomic(Real a, Real b, Real c, dou
     }
     __syncthreads();
     if (warp == 0) {
-        if constexpr (NW <= 8) {
+        if constexpr (NW % 8 == 0) {
             const int v = lane >> 3, w = lane & 7;
-            double d = (v < 3 && w < NW) ? (double)red_s[v < 3 ? v : 0][w < NW ? w : 0] : 0.0;
+            double d = 0.0;
+            if (v < 3)
+#pragma unroll
+                for (int k = 0; k < NW; k += 8) d += (double)red_s[v][w + k];
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
             if (w == 0 && v < 3) atomicAdd(out + v, d);

@@ -297,6 +297,27 @@ static size_t level_d_bytes(const dir_ctx* c, int l) {
            sizeof(float);
 }
 
+// Schedule 4: the whole level in one launch, its field resident in the shared
+// memory of a cluster (dir_level.cu).  Only where nothing looks in between the
+// iterations: no stop test, no timing events; and only by default (fuse = 2).
+static bool level_wants_resident(const dir_ctx* c, int l) {
+    return c->p.fuse == 2 && c->p.stop_mode == 0 && !c->p.timing && level_split_ok(c, l);
+}
+
+static dirk::LevelArgs level_args(const dir_ctx* c, int lc, int row, char* u) {
+    const int l = c->levels - 1 - lc;
+    dirk::LevelArgs a;
+    a.S = c->lv[l].S;
+    a.M = c->lv[l].M;
+    a.u = reinterpret_cast<float*>(u);
+    a.g = c->lv[l].g;
+    a.alpha2 = (float)(c->p.alpha * c->p.alpha);
+    a.red = c->red + 3 * (size_t)row;
+    a.corr = c->corr ? c->corr + 4 * (size_t)row : nullptr;
+    a.iters = c->p.iters[lc];
+    return a;
+}
+
 // The scratch of schedule 3 into the arguments of its two kernels: D, Eq. 6's d,
 // then u where the z + D kernel writes it (else both read t from their u)
 static void d_scratch(const dir_ctx* c, const Grid3& g, bool writes_u, dirk::ForceArgs& za,
@@ -321,6 +342,7 @@ static int level_schedule(const dir_ctx* c, int l) {
     if (c->fp64 || c->p.plain_kernels) return 0;
     const Grid3& g = c->lv[l].g;
     const bool split_ok = level_split_ok(c, l);
+    if (level_wants_resident(c, l) && dirk::level_resident(c->variant, g)) return 4;
     if (level_wants_d(c, l) && c->C && c->C_bytes >= level_d_bytes(c, l)) return 3;
     const bool eqs12 = c->variant == 0 || c->variant == 1;
     const bool fused_ok = c->p.stop_mode == 0 && dirk::fused_supported(c->variant) &&
@@ -488,6 +510,18 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
         const bool timed = c->p.timing && l == 0;
         const int n = c->p.iters[lc];
         const int sched = level_schedule(c, l);
+        if (sched == 4 && n > 0) {
+            dirk::LevelGroup G;
+            G.taps = c->taps;
+            G.cluster = dirk::level_cluster(&g, 1);
+            if (!dirk::level_group_add(G, c->variant, level_args(c, lc, row, cur)))
+                return DIR_EINVAL;
+            CK(c, dirk::launch_level(c->variant, c->img_type(l), G, s));
+            c->launches += 1;
+            row += n;
+            c->fused_level[lc] = 4;
+            continue;
+        }
         if (sched == 1 && n > 0) {
             // iteration 0 from u, iterations 1..n-1 from the previous v with the
             // smoothing folded in, then one smoothing of the last v
@@ -1234,9 +1268,10 @@ static bool batch_groupable(dir_ctx* const* ctxs, int n) {
 
 // Records one chunk of the grouped form on stream s (under capture): jobs of
 // one force law and image storage, at most kGroupMax, moving in lockstep.  Per
-// level: each job's field start and first force pass, then every later
-// iteration as one grouped x/y and one grouped z + force launch over all the
-// jobs, then each job's last smoothing.
+// level: each job's field start; then, for the jobs whose level a cluster
+// holds, one launch of a cluster each; for the others each job's first force
+// pass, every later iteration as one grouped x/y and one grouped z + force launch
+// over them, and each one's last smoothing.
 static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& jobs,
                                  cudaStream_t s) {
     const int n = (int)jobs.size();
@@ -1255,26 +1290,50 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
     for (int lc = 0; lc < L; ++lc) {
         const int l = L - 1 - lc;
         const int iters = c0->p.iters[lc];
-        std::vector<Grid3> grids(n);
         for (int q = 0; q < n; ++q) {
             dir_ctx* c = ctxs[jobs[q]];
             const int rc = enqueue_level_start(c, lc, cur[q], oth[q], s);
             if (rc != DIR_OK) return rc;
             c->level_first[lc] = row[q];
             c->fused_level[lc] = 0;
-            grids[q] = c->lv[l].g;
         }
         if (iters == 0) continue;
+        // jobs whose level a cluster holds: all their iterations in one launch;
+        // act: the others, in lockstep below
+        std::vector<int> act;
+        dirk::LevelGroup R;
+        R.taps = c0->taps;
+        std::vector<Grid3> held;
+        for (int q = 0; q < n; ++q)
+            if (level_schedule(ctxs[jobs[q]], l) == 4) held.push_back(ctxs[jobs[q]]->lv[l].g);
+        R.cluster = dirk::level_cluster(held.data(), (int)held.size());
+        for (int q = 0; q < n; ++q) {
+            dir_ctx* c = ctxs[jobs[q]];
+            if (level_schedule(c, l) != 4) {
+                act.push_back(q);
+                continue;
+            }
+            if (!dirk::level_group_add(R, c->variant, level_args(c, lc, row[q], cur[q])))
+                return DIR_EINVAL;
+            c->fused_level[lc] = 4;
+            c->launches += 1;
+            row[q] += iters;
+        }
+        if (R.n > 0) CK(c0, dirk::launch_level(c0->variant, c0->img_type(l), R, s));
+        if (act.empty()) continue;
+        const int na = (int)act.size();
+        std::vector<Grid3> grids(na);
+        for (int k = 0; k < na; ++k) grids[k] = ctxs[jobs[act[k]]]->lv[l].g;
         // Eqs. 3-6 where every job has its D scratch: the split after the
         // difference image, as each job's own registration would run it
         bool dform = c0->variant >= 2;
-        for (int q = 0; q < n; ++q) {
+        for (int q : act) {
             const dir_ctx* c = ctxs[jobs[q]];
             dform = dform && c->C && c->C_bytes >= level_d_bytes(c, l);
         }
-        for (int q = 0; q < n; ++q) ctxs[jobs[q]]->fused_level[lc] = dform ? 3 : 2;
+        for (int q : act) ctxs[jobs[q]]->fused_level[lc] = dform ? 3 : 2;
         // iteration 0 from the level's starting field, per job
-        for (int q = 0; q < n; ++q) {
+        for (int q : act) {
             dir_ctx* c = ctxs[jobs[q]];
             dirk::ForceArgs fa = level_force_args(c, lc);
             fa.u = cur[q];
@@ -1287,9 +1346,9 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             c->launches += 1;
         }
         long long chunk_vox = 0;  // the level of the whole chunk
-        for (int q = 0; q < n; ++q) chunk_vox += (long long)grids[q].nx * grids[q].ny * grids[q].nz;
+        for (const Grid3& g : grids) chunk_vox += (long long)g.nx * g.ny * g.nz;
         int boxes = 0, zc = 0, depth = 0;
-        dirk::group_shapes(c0->variant, grids.data(), n, c0->num_sms, &boxes, &zc, &depth);
+        dirk::group_shapes(c0->variant, grids.data(), na, c0->num_sms, &boxes, &zc, &depth);
         dirk::XYGroup X;
         dirk::ZSGroup Z;
         dirk::ZDGroup ZD;
@@ -1301,7 +1360,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
         Z.variant = ZD.variant = ST.variant = c0->variant;
         Z.depth = ZD.depth = ST.depth = depth;
         Z.taps = ZD.taps = ST.taps = c0->taps;
-        for (int q = 0; q < n; ++q) {
+        for (int q : act) {
             dir_ctx* c = ctxs[jobs[q]];
             dirk::SmoothArgs sa = level_smooth_args(c, lc);
             sa.in = oth[q];
@@ -1316,7 +1375,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             bool added = dirk::xy_group_add(X, sa);
             if (dform) {
                 dirk::ForceArgs za = fa, ta = fa;
-                d_scratch(c, grids[q], ZD.writes_u, za, ta);
+                d_scratch(c, c->lv[l].g, ZD.writes_u, za, ta);
                 added = added && dirk::d_group_add(ZD, ST, za, ta);
             } else {
                 added = added && dirk::zs_group_add(Z, fa);
@@ -1329,15 +1388,15 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
         const int img = c0->img_type(l);
         const bool pdl = c0->p.pdl && chunk_vox > (1LL << 18);
         for (int it = 1; it < iters; ++it) {
-            for (int q = 0; q < n; ++q) {
-                dir_ctx* c = ctxs[jobs[q]];
-                const size_t r = (size_t)(row[q] + it);
-                dirk::ForceArgs& fa = dform ? ST.a[q] : Z.a[q];
+            for (int k = 0; k < na; ++k) {
+                dir_ctx* c = ctxs[jobs[act[k]]];
+                const size_t r = (size_t)(row[act[k]] + it);
+                dirk::ForceArgs& fa = dform ? ST.a[k] : Z.a[k];
                 fa.red = c->red + 3 * r;
                 fa.corr = c->corr ? c->corr + 4 * r : nullptr;
                 fa.iter = it;
-                ZD.a[q].iter = it;
-                X.a[q].iter = it;
+                ZD.a[k].iter = it;
+                X.a[k].iter = it;
                 c->launches += dform ? 3 : 2;
             }
             CK(c0, dirk::launch_smooth_xy_grouped(X, s, pdl));
@@ -1347,7 +1406,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
                 CK(c0, dirk::launch_force_zs_grouped(c0->variant, img, Z, s, pdl));
         }
         // u = G v of the last iteration, per job
-        for (int q = 0; q < n; ++q) {
+        for (int q : act) {
             dir_ctx* c = ctxs[jobs[q]];
             dirk::SmoothArgs sa = level_smooth_args(c, lc);
             sa.in = oth[q];

@@ -177,6 +177,35 @@ bool d_group_add(ZDGroup& Z, STGroup& T, const ForceArgs& zd, const ForceArgs& s
 cudaError_t launch_force_d_grouped(int img_type, const ZDGroup& Z, const STGroup& T,
                                    cudaStream_t s, bool pdl = false);
 
+// All iterations of a small level in one launch, the field resident in the
+// shared memory of one thread-block cluster per volume (dir_level.cu; FP32 field,
+// float or int16 images, radius 3, no stop test): u is the level's starting field
+// and its result; red and corr the rows of its iterations, 3 and 4 doubles each.
+constexpr int kLevelCluster = 16;  // most CTAs of a cluster
+constexpr long long kLevelMaxVoxels = 16384;
+struct LevelArgs {
+    const void* S;
+    const void* M;
+    float* u;
+    Grid3 g;
+    float alpha2;
+    double* red;
+    double* corr;       // or null
+    int iters;
+    int tile_rows = 0, tile_planes = 0;  // set by level_group_add
+};
+struct LevelGroup {
+    LevelArgs a[kGroupMax];
+    Taps taps;
+    int n = 0;          // jobs, one cluster each (one force law, image storage, cluster size)
+    int cluster = 0;    // CTAs per cluster
+    int smem = 0;       // bytes per CTA
+};
+bool level_resident(int variant, const Grid3& g);  // small enough, and its tiles fit
+int level_cluster(const Grid3* g, int n);          // LevelGroup::cluster for these levels
+bool level_group_add(LevelGroup& G, int variant, const LevelArgs& a);
+cudaError_t launch_level(int variant, int img_type, const LevelGroup& G, cudaStream_t s);
+
 // One fused iteration (Eqs. 1-2 only): u = G_sigma * vin on the fly, then the
 // force kernel's work, v = u - dr(u); red as for ForceArgs.
 struct FusedArgs {

@@ -41,7 +41,10 @@ def test_production_kernels_equal_plain(dims, i16):
         # float images for the plain reference: whole numbers, so the same values
         ref, href = _run(dl, S.astype(np.float32), M.astype(np.float32), dims, variant, False,
                          plain_kernels=1)
-        for kw in ({}, {"correlation": 1, "pdl": 0}, {"stop_mode": 1, "eps": 0.0}):
+        # by default the whole level in one cluster launch (with and without the
+        # correlation sums), then the split kernels (fuse 3: Eqs. 3-6 in one pass)
+        for kw in ({}, {"correlation": 1}, {"fuse": 4, "pdl": 0}, {"fuse": 3},
+                   {"fuse": 4, "correlation": 1}, {"stop_mode": 1, "eps": 0.0}):
             u, h = _run(dl, S, M, dims, variant, i16, **kw)
             assert np.array_equal(u, ref, equal_nan=True), (variant, kw, np.abs(u - ref).max())
             # sums of n positive terms, rounded in FP32 within a thread and a
