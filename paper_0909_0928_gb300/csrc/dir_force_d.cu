@@ -139,20 +139,19 @@ int force_d_planes(int variant, const Grid3& g) {
     return (variant == 5 ? 2 : 1) + (force_d_writes_u(g) ? 3 : 0);
 }
 
-// Brick depth of the force pass (the z + D pass caps it): 8 where such bricks
-// still number four per SM, else the deepest of 4 and 2 that gives one per SM,
-// else 1.  Eq. 6 on large levels takes 4: with its d box, 8 leaves three blocks
-// per SM (256x256x100: 113.4 us per iteration at 4, 119 at 8; Eq. 3 the other
-// way round, 100.8 and 97.9).  Blocks per SM there: five of the z + D kernel for
-// Eqs. 3-5 (95.9 us per iteration against 97.9 with four), four for Eq. 6 (119
-// against 122: its two interpolations want the registers).
+// Brick depth of the force pass (the z + D pass caps it at 4): 8 for Eqs. 3-5
+// where such bricks number three per SM, else 4 where those number one per SM,
+// else 2.  Measured per iteration with the force pass at 2 / 4 / 8, Eq. 3: 48x48x24
+// 7.7 / 8.0 / 8.5 us, 64x64x25 7.95 / 7.81 / 8.40, 96x96x48 13.6 / 12.9 / 13.4,
+// 128x128x64 21.6 / 20.7 / 19.8.  Eq. 6 stays at 4: with its d box, 8 leaves three
+// blocks per SM (128x128x64 23.7 against 23.9; 256x256x100 113.4 against 119).
+// Blocks per SM on large levels: five of the z + D kernel for Eqs. 3-5 (95.9 us per
+// iteration at 256x256x100 against 97.9 with four), four for Eq. 6 (119 against 122:
+// its two interpolations want the registers).
 int force_d_depth(int variant, const Grid3& g, int num_sms) {
     const long long bxy = (long long)((g.nx + FTX - 1) / FTX) * ((g.ny + FTY - 1) / FTY);
-    if (variant == 5 && !force_d_writes_u(g)) return 4;
-    if (bxy * ((g.nz + 7) / 8) >= 4LL * num_sms) return 8;
-    for (int d = 4; d >= 2; d /= 2)
-        if (bxy * ((g.nz + d - 1) / d) >= num_sms) return d;
-    return 1;
+    if (variant != 5 && bxy * ((g.nz + 7) / 8) >= 3LL * num_sms) return 8;
+    return bxy * ((g.nz + 3) / 4) >= num_sms ? 4 : 2;
 }
 
 cudaError_t launch_force_d(int variant, const ForceArgs& zd, const ForceArgs& st, const Taps& taps,

@@ -135,15 +135,22 @@ static cudaError_t launch_gzs_types(int variant, const ForceArgs& a, const Taps&
     }
 }
 
-// Brick depth: Eq. 1 takes 6 planes where that still gives four waves of
-// blocks -- the brick of t with its 2R halo planes and the S box then fit four
-// blocks per SM in shared memory instead of three (measured on 256x256x100:
-// 65.4 us against 70.3 us at depth 8); otherwise, and for Eq. 2 with its M box,
-// the force pass's usual depth.
+// Brick depth.  Large levels: Eq. 1 takes 6 planes (four blocks per SM, as at 4,
+// with less halo), Eq. 2 with its M box 4 (6 and 8 leave three blocks per SM).
+// Below 16 six-plane bricks per SM: 4 planes while those number two per SM, else
+// 2; but where four-plane bricks are just over one wave of resident blocks, the
+// shallowest brick that makes it one wave.  Measured per iteration at depths
+// 2 / 4 / 6 / 8, Eq. 1 and Eq. 2:
+//   256x256x100  86.7 / 73.4 / 73.0 / 80.0 us    91.2 / 76.0 / 85.7 / 89.2
+//   193x171x87   48.4 / 41.7 / 42.1 / 44.9       51.0 / 43.2 / 48.5 / 49.9
+//   128x128x64   17.7 / 16.4 / 17.2 / 18.1       18.6 / 17.0 / 19.3 / 20.8
+//   128x128x50   15.6 / 14.8 / 14.2 / 14.4       15.8 / 16.9 / 18.6 / 15.8
+//   96x96x48     11.5 / 10.4 / 10.7 / 11.6       12.1 / 11.1 / 11.6 / 13.3
+//   96x96x24      7.2 /  7.8 /  8.0 /  8.6        7.6 /  8.2 /  8.7 / 10.3
+//   48x48x24      5.5 /  6.3 /  7.2 /  7.8 (1: 5.7)
 int force_zs_depth(int variant, const Grid3& g, int num_sms) {
     const long long bxy = (long long)((g.nx + FTX - 1) / FTX) * ((g.ny + FTY - 1) / FTY);
-    if (variant == 0 && bxy * ((g.nz + 5) / 6) >= 4LL * 4 * num_sms) return 6;
-    return force_brick_depth(g, num_sms);
+    return force_zs_depth_of(variant, num_sms, [&](int d) { return bxy * ((g.nz + d - 1) / d); });
 }
 
 bool force_zs_supported(int variant, const ForceArgs& a, const Taps& taps) {

@@ -108,12 +108,12 @@ void group_shapes(int variant, const Grid3* grids, int n, int num_sms, int* boxe
                  ((grids[j].nz + d - 1) / d);
         return b;
     };
-    if (variant == 0 && bricks(6) >= 4LL * 4 * num_sms) {
-        *depth = 6;
+    if (variant <= 1) {
+        *depth = force_zs_depth_of(variant, num_sms, bricks);
         return;
     }
     *depth = 1;
-    for (int d = variant >= 2 ? 4 : 8; d > 1; d /= 2)
+    for (int d = 4; d > 1; d /= 2)
         if (bricks(d) >= num_sms) {
             *depth = d;
             break;

@@ -84,6 +84,17 @@ cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s);
 // launch_smooth + launch_force.  Brick depth a.depth (8, 6, 4, 2 or 1).
 bool force_zs_supported(int variant, const ForceArgs& a, const Taps& taps);
 int force_zs_depth(int variant, const Grid3& g, int num_sms);
+// its rule on any count of bricks by depth (Eqs. 1-2; a group of volumes)
+template <typename Bricks>
+int force_zs_depth_of(int variant, int num_sms, Bricks&& bricks) {
+    if (bricks(6) >= 16LL * num_sms) return variant == 0 ? 6 : 4;
+    if (bricks(4) < 2LL * num_sms) return 2;
+    const long long wave = 4LL * num_sms;  // resident four-plane bricks
+    if (bricks(4) > wave && 2 * bricks(4) < 3 * wave)
+        for (int d = 6; d <= 8; d += 2)  // resident: 4 per SM of Eq. 1's at 6, else 3
+            if (bricks(d) <= (variant == 0 && d == 6 ? 4LL : 3LL) * num_sms) return d;
+    return 4;
+}
 cudaError_t launch_force_zs(int variant, const ForceArgs& a, const Taps& taps, cudaStream_t s);
 
 // Eqs. 3-6, the split iteration with the difference image formed once per
