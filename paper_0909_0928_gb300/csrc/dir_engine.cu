@@ -297,6 +297,9 @@ static size_t level_d_bytes(const dir_ctx* c, int l) {
            sizeof(float);
 }
 
+// The interleaved mid-space field of Eq. 6's output step, in the scratch too
+static size_t ic_bytes(const dir_ctx* c) { return 4 * sizeof(float) * (size_t)c->lv[0].g.cs; }
+
 // Schedule 4: the whole level in one launch, its field resident in the shared
 // memory of a cluster (dir_level.cu).  Only where nothing looks in between the
 // iterations: no stop test, no timing events; and only by default (fuse = 2).
@@ -476,8 +479,16 @@ static dirk::SmoothArgs level_smooth_args(const dir_ctx* c, int lc) {
 // inverse-consistent law, and where the result lives.
 static int enqueue_epilogue(dir_ctx* c, char* cur, char* oth, cudaStream_t s) {
     if (c->variant == DIR_INVERSE_CONSISTENT) {
-        CK(c, dirk::launch_ic_invert(c->fp64, c->field_type, cur, oth, c->lv[0].g, kIcInvertSteps, s));
-        c->launches += 1;
+        const Grid3& g = c->lv[0].g;
+        if (level_wants_d(c, 0) && dirk::ic_invert4_supported(g) && c->C &&
+            c->C_bytes >= ic_bytes(c)) {
+            CK(c, dirk::launch_ic_invert4(reinterpret_cast<const float*>(cur), c->C,
+                                          reinterpret_cast<float*>(oth), g, kIcInvertSteps, s));
+            c->launches += 2;
+        } else {
+            CK(c, dirk::launch_ic_invert(c->fp64, c->field_type, cur, oth, g, kIcInvertSteps, s));
+            c->launches += 1;
+        }
         c->final_field = oth;
     } else {
         c->final_field = cur;
@@ -897,6 +908,9 @@ int dir_create(dir_ctx** out, const void* static_img, const void* moving_img, co
     for (int l = 0; l < c->levels; ++l)
         if (p.iters[c->levels - 1 - l] > 0 && level_wants_d(c, l))
             c->C_bytes = std::max(c->C_bytes, level_d_bytes(c, l));
+    if (c->variant == DIR_INVERSE_CONSISTENT && level_wants_d(c, 0) &&
+        dirk::ic_invert4_supported(c->lv[0].g))
+        c->C_bytes = std::max(c->C_bytes, ic_bytes(c));
     if (c->C_bytes > 0 && cudaMallocAsync(&c->C, c->C_bytes, st) != cudaSuccess) {
         cudaGetLastError();
         g_create_error = "device allocation failed";

@@ -249,6 +249,11 @@ cudaError_t launch_upsample(bool fp64, int ftype, const void* coarse, const Grid
 // out(x) = img(x + u(x)); img in the arithmetic type, out written dense float
 cudaError_t launch_warp(bool fp64, int ftype, const void* img, const void* u, const Grid3& g,
                         float* out_dense, cudaStream_t s);
+// launch_ic_invert in single precision by way of an interleaved copy of h (scratch:
+// 4 * g.cs floats); two kernels
+bool ic_invert4_supported(const Grid3& g);
+cudaError_t launch_ic_invert4(const float* h, void* scratch, float* u, const Grid3& g, int steps,
+                              cudaStream_t s);
 // u(y) = 2 h(x*), x* = y + h(x*) by `steps` fixed-point steps (Eq. 6 output)
 cudaError_t launch_ic_invert(bool fp64, int ftype, const void* h, void* u, const Grid3& g,
                              int steps, cudaStream_t s);

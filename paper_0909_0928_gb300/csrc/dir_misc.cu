@@ -7,6 +7,7 @@
 
 #include "dir_common.cuh"
 #include "dir_launch.h"
+#include "dir_pair.cuh"
 
 namespace dirk {
 
@@ -78,6 +79,80 @@ __global__ void ic_invert_kernel(const TF* __restrict__ h, TF* __restrict__ u, G
     u[o] = st_as<TF>(Real(2) * trilinear<Real>(hx, g, x, ax, y, ay, z, az));
     u[o + g.cs] = st_as<TF>(Real(2) * trilinear<Real>(hy, g, x, ax, y, ay, z, az));
     u[o + 2 * g.cs] = st_as<TF>(Real(2) * trilinear<Real>(hz, g, x, ax, y, ay, z, az));
+}
+
+// The same in single precision from an interleaved copy of h, {hx, hy, hz, 0} per
+// voxel: a corner is one 16-byte load instead of three loads, its address and
+// weights are found once for the three components, x and y are lerped as a packed
+// pair, and the corners stay in registers while a stays in their cell (it leaves it
+// in the first few steps only).  256x256x100: 1398 us with ic_invert_kernel, 372 +
+// 31 for the copy here (520 with the corners loaded at every step), now bound by
+// its arithmetic: 78 instructions a step, 76% of the issue rate.
+__global__ void interleave_kernel(const float* __restrict__ h, Grid3 g, float4* __restrict__ q) {
+    const int x = blockIdx.x * MTX + threadIdx.x, y = blockIdx.y * MTY + threadIdx.y;
+    if (x >= g.nx || y >= g.ny) return;
+    const int o = offs(g, x, y, blockIdx.z);
+    q[o] = make_float4(h[o], h[o + g.cs], h[o + 2 * g.cs], 0.0f);
+}
+
+struct Lerp3 {
+    f32x2 xy;
+    float z;
+};
+__device__ __forceinline__ Lerp3 lerp3(const Lerp3& a, const Lerp3& b, float f) {
+    const float g = 1.0f - f;
+    return {f2_fma(b.xy, f2_dup(f), f2_mul(a.xy, f2_dup(g))), fmaf(b.z, f, __fmul_rn(a.z, g))};
+}
+
+__global__ void __launch_bounds__(MTX * MTY)
+    ic_invert4_kernel(const float4* __restrict__ h, float* __restrict__ u, Grid3 g, int steps) {
+    const int x = blockIdx.x * MTX + threadIdx.x, y = blockIdx.y * MTY + threadIdx.y;
+    const int z = blockIdx.z;
+    if (x >= g.nx || y >= g.ny) return;
+    const AxisBounds bx((float)x, g.nx - 1, max(g.nx - 2, 0)),
+        by((float)y, g.ny - 1, max(g.ny - 2, 0)), bz((float)z, g.nz - 1, max(g.nz - 2, 0));
+    const uint32_t px = 16u * g.px, pl = 16u * (uint32_t)g.plane;
+    const uint32_t sx = g.nx > 1 ? 16u : 0u, sy = g.ny > 1 ? px : 0u, sz = g.nz > 1 ? pl : 0u;
+    const int o = offs(g, x, y, z);
+    const uint32_t o0 = 16u * (uint32_t)o - kMagicBits * (16u + px + pl);
+    auto corner = [](float off, const AxisBounds& b, float& f) {  // as pair_corner, one lane
+        const float c = r_clamp(off, b.lo, b.hi);
+        const float t = fminf(__fadd_rd(c, kMagic), b.top);
+        f = c - (t - kMagic);
+        return __float_as_uint(t);
+    };
+    uint32_t held = ~0u;  // byte offset of the cell whose corners c holds (a multiple of 16)
+    Lerp3 c[8];
+    auto at = [&](float ax, float ay, float az) {  // h at (x, y, z) + a
+        float fx, fy, fz;
+        const uint32_t p = o0 + 16u * corner(ax, bx, fx) + px * corner(ay, by, fy) +
+                           pl * corner(az, bz, fz);
+        if (p != held) {
+            held = p;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float4 v = __ldg(
+                    at_byte(h, p + (k & 1 ? sx : 0u) + (k & 2 ? sy : 0u) + (k & 4 ? sz : 0u)));
+                c[k] = Lerp3{f2_pack(v.x, v.y), v.z};
+            }
+        }
+        const Lerp3 v0 = lerp3(lerp3(c[0], c[1], fx), lerp3(c[2], c[3], fx), fy);
+        const Lerp3 v1 = lerp3(lerp3(c[4], c[5], fx), lerp3(c[6], c[7], fx), fy);
+        return lerp3(v0, v1, fz);
+    };
+    float ax = 0.0f, ay = 0.0f, az = 0.0f;
+    for (int s = 0; s < steps; ++s) {
+        const Lerp3 n = at(ax, ay, az);
+        const bool fixed = f2_lo(n.xy) == ax && f2_hi(n.xy) == ay && n.z == az;
+        ax = f2_lo(n.xy);
+        ay = f2_hi(n.xy);
+        az = n.z;
+        if (fixed) break;
+    }
+    const Lerp3 r = at(ax, ay, az);
+    u[o] = 2.0f * f2_lo(r.xy);
+    u[o + g.cs] = 2.0f * f2_hi(r.xy);
+    u[o + 2 * g.cs] = 2.0f * r.z;
 }
 
 template <typename Real, typename TF, typename Out>
@@ -167,6 +242,19 @@ cudaError_t launch_warp(bool fp64, int ftype, const void* img, const void* u, co
     DIR_DISPATCH_F(fp64, ftype, (warp_kernel<Real, TF><<<grid_for(g), dim3(MTX, MTY), 0, s>>>(
                                     static_cast<const Real*>(img), static_cast<const TF*>(u), g,
                                     out_dense)));
+    return cudaGetLastError();
+}
+
+bool ic_invert4_supported(const Grid3& g) { return g.cs < (1LL << 28); }  // 32-bit byte offsets
+
+cudaError_t launch_ic_invert4(const float* h, void* scratch, float* u, const Grid3& g, int steps,
+                              cudaStream_t s) {
+    if (!ic_invert4_supported(g)) return cudaErrorInvalidValue;
+    float4* q = static_cast<float4*>(scratch);
+    interleave_kernel<<<grid_for(g), dim3(MTX, MTY), 0, s>>>(h, g, q);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    ic_invert4_kernel<<<grid_for(g), dim3(MTX, MTY), 0, s>>>(q, u, g, steps);
     return cudaGetLastError();
 }
 

@@ -90,6 +90,10 @@ template <typename T>
 __device__ __forceinline__ T* at_byte(T* base, uint32_t byte) {
     return reinterpret_cast<T*>(reinterpret_cast<char*>(base) + byte);
 }
+template <typename T>
+__device__ __forceinline__ const T* at_byte(const T* base, uint32_t byte) {
+    return reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + byte);
+}
 
 // Corner search along one axis for a pair of voxels, bounds as floats: p is
 // clamped to [0, n - 1] in offset form (lo = -base, hi = n - 1 - base), its
