@@ -388,6 +388,14 @@ static int enqueue_prologue(dir_ctx* c, cudaStream_t s) {
         const Grid3& gf = c->lv[l - 1].g;
         const Grid3& gc = c->lv[l].g;
         for (int img = 0; img < 2; ++img) {
+            if (!f64 && !plain) {
+                const char* in = img ? c->lv[l - 1].M : c->lv[l - 1].S;
+                char* out = img ? c->lv[l].M : c->lv[l].S;
+                CK(c, dirk::launch_pyramid(c->img_type(l - 1), in, gf, reinterpret_cast<float*>(c->B),
+                                           reinterpret_cast<float*>(out), gc, c->taps1, s));
+                c->launches += 2;
+                continue;
+            }
             dirk::SmoothArgs sa;
             sa.in = img ? c->lv[l - 1].M : c->lv[l - 1].S;
             sa.out = c->B;

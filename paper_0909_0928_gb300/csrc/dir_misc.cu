@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "dir_common.cuh"
 #include "dir_launch.h"
 #include "dir_pair.cuh"
@@ -26,19 +28,73 @@ __global__ void decimate_kernel(const Real* __restrict__ in, Grid3 gi, Real* __r
     out[offs(go, x, y, z)] = __ldg(in + offs(gi, 2 * x, 2 * y, 2 * z));
 }
 
+// fine(x) = 2 * trilinear(coarse, x / 2).  A thread makes the 2 x 2 x 2 fine
+// voxels of one coarse cell from its eight corners (24 loads for 24 values; a
+// thread per fine voxel gathered 24 per three values: 55.7 us at 256x256x100, now
+// 21).
+// The lerps and their weights are those of `trilinear`: along each axis the even
+// voxel sits on the cell's corner (weight 0) and the odd one half way; past the
+// last corner both clamp to it (weight 1 from the corner before).
 template <typename Real, typename TF>
 __global__ void upsample_kernel(const TF* __restrict__ coarse, Grid3 gc, TF* __restrict__ fine,
                                 Grid3 gf) {
-    const int x = blockIdx.x * MTX + threadIdx.x, y = blockIdx.y * MTY + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= gf.nx || y >= gf.ny) return;
-    // coarse position x / 2 = (x >> 1) + (x & 1) / 2, exact
-    const Real hx = Real(0.5) * (x & 1), hy = Real(0.5) * (y & 1), hz = Real(0.5) * (z & 1);
-    const long long o = (long long)offs(gf, x, y, z);
+    const int X = blockIdx.x * MTX + threadIdx.x, Y = blockIdx.y * MTY + threadIdx.y;
+    const int Z = blockIdx.z;
+    if (X >= gc.nx || Y >= gc.ny) return;
+    auto axis = [](int i, int n, int& i0, int& i1, Real (&f)[2]) {
+        const bool last = i >= n - 1;
+        i0 = n < 2 ? 0 : (last ? n - 2 : i);
+        i1 = n < 2 ? 0 : i0 + 1;
+        f[0] = (last && n > 1) ? Real(1) : Real(0);
+        f[1] = n < 2 ? Real(0) : (last ? Real(1) : Real(0.5));
+    };
+    int x0, x1, y0, y1, z0, z1;
+    Real fx[2], fy[2], fz[2];
+    axis(X, gc.nx, x0, x1, fx);
+    axis(Y, gc.ny, y0, y1, fy);
+    axis(Z, gc.nz, z0, z1, fz);
+    const int r[4] = {offs(gc, 0, y0, z0), offs(gc, 0, y1, z0), offs(gc, 0, y0, z1),
+                      offs(gc, 0, y1, z1)};
+    const int ofine = offs(gf, 2 * X, 2 * Y, 2 * Z);
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-        fine[o + c * gf.cs] = st_as<TF>(
-            Real(2) * trilinear<Real>(coarse + c * gc.cs, gc, x >> 1, hx, y >> 1, hy, z >> 1, hz));
+    for (int c = 0; c < 3; ++c) {
+        const TF* p = coarse + c * gc.cs;
+        TF* q = fine + c * gf.cs;
+        Real rx[4][2];  // the four rows lerped along x, even and odd
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const Real a = ldg_as<Real>(p + r[k] + x0), b = ldg_as<Real>(p + r[k] + x1);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) rx[k][i] = r_fma(b, fx[i], a * (Real(1) - fx[i]));
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (2 * Y + j >= gf.ny) break;
+            Real v0[2], v1[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                v0[i] = r_fma(rx[1][i], fy[j], rx[0][i] * (Real(1) - fy[j]));
+                v1[i] = r_fma(rx[3][i], fy[j], rx[2][i] * (Real(1) - fy[j]));
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (2 * Z + k >= gf.nz) break;
+                TF o[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    o[i] = st_as<TF>(Real(2) * r_fma(v1[i], fz[k], v0[i] * (Real(1) - fz[k])));
+                TF* d = q + ofine + j * gf.px + k * (int)gf.plane;
+                if constexpr (std::is_same<TF, float>::value) {
+                    if (2 * X + 1 < gf.nx) {
+                        *reinterpret_cast<float2*>(d) = make_float2(o[0], o[1]);
+                        continue;
+                    }
+                }
+                d[0] = o[0];
+                if (2 * X + 1 < gf.nx) d[1] = o[1];
+            }
+        }
+    }
 }
 
 template <typename Real, typename TF>
@@ -181,6 +237,55 @@ __global__ void import_kernel(const float* __restrict__ dense, TF* __restrict__ 
     for (int c = 0; c < ncomp; ++c) f[o + c * g.cs] = st_as<TF>((Real)dense[d + c * n]);
 }
 
+// One pyramid step (Sec. 2.3) of an image in single precision: the unit Gaussian
+// (radius 3) evaluated only where the coarser level samples it, in two kernels:
+// the x and y passes at even columns and rows of every plane, then the z pass at
+// even planes.  Taps oldest first, fused multiply-adds from zero, as the
+// smoothing kernels.  Smoothing the whole image and then sampling it took 27.6 +
+// 5.2 us per 256x256x100 image (int16: 37.0 + 5.0), now 17.0 + 5.6.
+constexpr int PR = 3;
+template <typename TI>
+__global__ void __launch_bounds__(MTX * MTY)
+    pyramid_xy_kernel(const TI* __restrict__ in, Grid3 gi, float* __restrict__ t, Grid3 go,
+                      const Taps taps) {
+    constexpr int ROWS = 2 * MTY + 2 * PR - 1;  // fine rows 2 Y0 - 3 .. 2 (Y0 + 7) + 3
+    __shared__ float xf[ROWS][MTX];
+    const int tx = threadIdx.x, ty = threadIdx.y, z = blockIdx.z;
+    const int X = blockIdx.x * MTX + tx, Y0 = blockIdx.y * MTY;
+    const TI* plane = in + (size_t)gi.plane * z;
+    for (int r = ty; r < ROWS; r += MTY) {
+        const TI* row = plane + (size_t)gi.px * clampi(2 * Y0 - PR + r, 0, gi.ny - 1);
+        float acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 2 * PR + 1; ++k)
+            acc = fmaf(taps.wf[k <= PR ? k : 2 * PR - k],
+                       ldg_as<float>(row + clampi(2 * X - PR + k, 0, gi.nx - 1)), acc);
+        xf[r][tx] = acc;
+    }
+    __syncthreads();
+    const int Y = Y0 + ty;
+    if (X >= go.nx || Y >= go.ny) return;
+    float acc = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 2 * PR + 1; ++k)
+        acc = fmaf(taps.wf[k <= PR ? k : 2 * PR - k], xf[2 * ty + k][tx], acc);
+    t[(size_t)go.plane * z + (size_t)go.px * Y + X] = acc;
+}
+
+__global__ void pyramid_z_kernel(const float* __restrict__ t, int nz, float* __restrict__ out,
+                                 Grid3 go, const Taps taps) {
+    const int X = blockIdx.x * MTX + threadIdx.x, Y = blockIdx.y * MTY + threadIdx.y;
+    const int Z = blockIdx.z;
+    if (X >= go.nx || Y >= go.ny) return;
+    const float* col = t + (size_t)go.px * Y + X;
+    float acc = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 2 * PR + 1; ++k)
+        acc = fmaf(taps.wf[k <= PR ? k : 2 * PR - k],
+                   __ldg(col + (size_t)go.plane * clampi(2 * Z - PR + k, 0, nz - 1)), acc);
+    out[offs(go, X, Y, Z)] = acc;
+}
+
 // Sec. 2.4: l(t) = sum|du| / sum|u|; stop the level after iteration t when
 // |l(t) - l(t - window)| <= eps (both defined).  One thread.
 __global__ void stop_test_kernel(const double* __restrict__ red, const double* __restrict__ corr,
@@ -232,7 +337,7 @@ cudaError_t launch_decimate(bool fp64, const void* in, const Grid3& gin, void* o
 
 cudaError_t launch_upsample(bool fp64, int ftype, const void* coarse, const Grid3& gc, void* fine,
                             const Grid3& gf, cudaStream_t s) {
-    DIR_DISPATCH_F(fp64, ftype, (upsample_kernel<Real, TF><<<grid_for(gf), dim3(MTX, MTY), 0, s>>>(
+    DIR_DISPATCH_F(fp64, ftype, (upsample_kernel<Real, TF><<<grid_for(gc), dim3(MTX, MTY), 0, s>>>(
                                     static_cast<const TF*>(coarse), gc, static_cast<TF*>(fine), gf)));
     return cudaGetLastError();
 }
@@ -255,6 +360,25 @@ cudaError_t launch_ic_invert4(const float* h, void* scratch, float* u, const Gri
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     ic_invert4_kernel<<<grid_for(g), dim3(MTX, MTY), 0, s>>>(q, u, g, steps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pyramid(int in_type, const void* in, const Grid3& gin, float* scratch,
+                           float* out, const Grid3& gout, const Taps& taps, cudaStream_t s) {
+    if (taps.R != PR) return cudaErrorInvalidValue;
+    dim3 grid = grid_for(gout);
+    grid.z = gin.nz;
+    if (in_type == kStoreF32)
+        pyramid_xy_kernel<float><<<grid, dim3(MTX, MTY), 0, s>>>(static_cast<const float*>(in), gin,
+                                                                 scratch, gout, taps);
+    else if (in_type == kStoreI16)
+        pyramid_xy_kernel<int16_t><<<grid, dim3(MTX, MTY), 0, s>>>(static_cast<const int16_t*>(in),
+                                                                   gin, scratch, gout, taps);
+    else
+        return cudaErrorInvalidValue;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    pyramid_z_kernel<<<grid_for(gout), dim3(MTX, MTY), 0, s>>>(scratch, gin.nz, out, gout, taps);
     return cudaGetLastError();
 }
 

@@ -50,3 +50,47 @@ def test_production_kernels_equal_plain(dims, i16):
             # sums of n positive terms, rounded in FP32 within a thread and a
             # warp and in FP64 beyond: at most 8 voxels and 32 threads deep
             np.testing.assert_allclose(h, href, rtol=64 * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2), (33, 9, 13), (40, 1, 9), (1, 9, 9), (97, 40, 1),
+                                  (64, 31, 26)], ids=lambda d: "x".join(map(str, d)))
+@pytest.mark.parametrize("i16", [False, True], ids=["f32", "i16"])
+def test_pyramid_and_upsampling(dims, i16):
+    """Two and three levels equal the plain kernels' pyramid; the upsampled field
+    is twice the trilinear interpolation of its own even voxels (weight 0: the
+    coarse values, exactly).  Three lerps of three roundings each, of values up
+    to the largest: 9 eps."""
+    import paper_0909_0928_gb300 as dl
+
+    S = np.round(400.0 * random_volume(dims, 21)).astype(np.int16 if i16 else np.float32)
+    M = np.round(400.0 * random_volume(dims, 22)).astype(S.dtype)
+
+    def run(a, b, dt, **kw):
+        p = dl.dir_params_default(alpha=0.7, **kw)
+        ctx = dl.dir_create(a, b, dims, (1.0, 1.0, 1.0), dt, False, 5, p)
+        try:
+            dl.dir_register(ctx)
+            u = np.empty((3,) + dims[::-1], np.float32)
+            return dl.dir_get_field(ctx, u)
+        finally:
+            dl.dir_destroy(ctx)
+
+    for levels, iters in ((2, [3, 2]), (3, [2, 1, 2])):
+        u = run(S, M, dl.DIR_I16 if i16 else dl.DIR_F32, levels=levels, iters=iters)
+        ref = run(S.astype(np.float32), M.astype(np.float32), dl.DIR_F32, levels=levels,
+                  iters=iters, plain_kernels=1)
+        assert np.array_equal(u, ref, equal_nan=True), np.abs(u - ref).max()
+
+    p = dl.dir_params_default(levels=2, iters=[4, 0], alpha=0.7)
+    ctx = dl.dir_create(S, M, dims, (1.0, 1.0, 1.0), dl.DIR_I16 if i16 else dl.DIR_F32, False, 0, p)
+    dl.dir_register(ctx)
+    f = dl.dir_get_field(ctx, np.empty((3,) + dims[::-1], np.float32)).astype(np.float64)
+    dl.dir_destroy(ctx)
+    want = f[:, ::2, ::2, ::2]
+    for axis, n in ((1, dims[2]), (2, dims[1]), (3, dims[0])):
+        pos = np.minimum(np.arange(n) / 2, want.shape[axis] - 1)
+        lo = np.floor(pos).astype(int)
+        hi = np.minimum(lo + 1, want.shape[axis] - 1)
+        w = (pos - lo).reshape([-1 if a == axis else 1 for a in range(4)])
+        want = want.take(lo, axis) * (1 - w) + want.take(hi, axis) * w
+    assert np.abs(f - want).max() <= 9 * 2.0 ** -24 * np.abs(f).max()
