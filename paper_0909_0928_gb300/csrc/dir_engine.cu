@@ -16,6 +16,8 @@
 // Single precision runs the TMA-tiled production kernels, or with
 // plain_kernels the plain-load kernels; double precision runs the plain-load
 // kernels in double.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -197,6 +199,34 @@ static int ensure(dir_ctx* c, void** p, size_t bytes) {
     return DIR_OK;
 }
 
+// Whether kernels of this device may read the caller's bytes [p, p + bytes): plain
+// memory of the device, the range inside one allocation.  What is not (another
+// device's memory, managed memory, a range past the allocation's end) stays with
+// the copies, which handle or refuse it.
+static bool device_readable(const void* p, size_t bytes, int device) {
+    static PFN_cuPointerGetAttributes_v7000 query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault,
+                                             &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(f);
+    }();
+    unsigned type = 0, managed = 0;
+    int ordinal = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* got[5] = {&type, &managed, &ordinal, &start, &size};
+    const CUdeviceptr a = (CUdeviceptr)(uintptr_t)p;
+    return query && query(5, what, got, a) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
+           !managed && ordinal == device && a >= start && bytes <= size && a - start <= size - bytes;
+}
+
 // Dense volume(s) (host or device) of element size src_esz (4 = float,
 // 2 = int16) -> pitched volume(s) of storage type dst_type.  Same element type:
 // a 2-D copy (exact); float -> bf16 / double: through the import kernel.
@@ -208,12 +238,18 @@ static int import_dense(dir_ctx* c, const void* src, int on_device, int src_esz,
                       (src_esz == 2 && dst_type == dirk::kStoreI16);
     if (same) {
         const size_t w = (size_t)g.nx * src_esz;
-        for (int comp = 0; comp < ncomp; ++comp)
-            CK(c, cudaMemcpy2DAsync(dst + comp * g.cs * dst_esz, (size_t)g.px * dst_esz,
-                                    static_cast<const char*>(src) + comp * n * src_esz, w, w,
+        for (int comp = 0; comp < ncomp; ++comp) {
+            const char* from = static_cast<const char*>(src) + comp * n * src_esz;
+            if (on_device && dirk::pitch_rows_supported(from, src_esz) &&
+                device_readable(from, n * src_esz, c->device)) {
+                CK(c, dirk::launch_pitch_rows(from, dst + comp * g.cs * dst_esz, g, src_esz, s));
+                continue;
+            }
+            CK(c, cudaMemcpy2DAsync(dst + comp * g.cs * dst_esz, (size_t)g.px * dst_esz, from, w, w,
                                     (size_t)g.ny * g.nz,
                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                     s));
+        }
         return DIR_OK;
     }
     if (src_esz != 4) return DIR_EUNSUPPORTED;
@@ -1156,18 +1192,38 @@ int dir_warp(dir_ctx* c, const void* img_in, void* img_out, dir_dtype dt, int on
     if (!c->have_field || !c->final_field) return DIR_ESTATE;
     const Grid3& g = c->lv[0].g;
     const size_t n = c->nvox();
-    int rc = ensure(c, (void**)&c->stage_img, (size_t)g.cs * c->esz);
-    if (rc != DIR_OK) return rc;
-    rc = import_dense(c, img_in, on_device, 4, c->stage_img, c->real_type, g, 1, c->stream);
-    if (rc != DIR_OK) return rc;
+    // a device image is gathered from where it lies, unless the output overlaps it
+    // (the copy of it was 26 MB and 60 us of a call at 256x256x100)
+    const bool pair = c->field_type == dirk::kStoreF32 && g.nx > 1;
+    const uintptr_t from = (uintptr_t)img_in, to = (uintptr_t)img_out;
+    const bool direct = pair && on_device && from % sizeof(float) == 0 &&
+                        (from + n * sizeof(float) <= to || to + n * sizeof(float) <= from) &&
+                        device_readable(img_in, n * sizeof(float), c->device);
+    int rc = DIR_OK;
+    Grid3 gi = g;
+    if (direct) {
+        gi.px = g.nx;
+        gi.plane = (long long)g.nx * g.ny;
+    } else {
+        rc = ensure(c, (void**)&c->stage_img, (size_t)g.cs * c->esz);
+        if (rc != DIR_OK) return rc;
+        rc = import_dense(c, img_in, on_device, 4, c->stage_img, c->real_type, g, 1, c->stream);
+        if (rc != DIR_OK) return rc;
+    }
     float* dst = (float*)img_out;
     if (!on_device) {
         rc = ensure(c, (void**)&c->stage_f32, 3 * n * sizeof(float));
         if (rc != DIR_OK) return rc;
         dst = c->stage_f32;
     }
-    CK(c, dirk::launch_warp(c->fp64, c->field_type, c->stage_img, c->final_field, g, dst,
-                            c->stream));
+    if (pair)
+        CK(c, dirk::launch_warp_pair(direct ? static_cast<const float*>(img_in)
+                                            : reinterpret_cast<const float*>(c->stage_img),
+                                     gi, reinterpret_cast<const float*>(c->final_field), g, dst,
+                                     c->stream));
+    else
+        CK(c, dirk::launch_warp(c->fp64, c->field_type, c->stage_img, c->final_field, g, dst,
+                                c->stream));
     if (!on_device)
         CK(c, cudaMemcpyAsync(img_out, dst, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));

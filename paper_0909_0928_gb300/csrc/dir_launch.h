@@ -249,10 +249,17 @@ cudaError_t launch_upsample(bool fp64, int ftype, const void* coarse, const Grid
 // out(x) = img(x + u(x)); img in the arithmetic type, out written dense float
 cudaError_t launch_warp(bool fp64, int ftype, const void* img, const void* u, const Grid3& g,
                         float* out_dense, cudaStream_t s);
+// the same in single precision, img on a grid of its own (px, plane), nx >= 2
+cudaError_t launch_warp_pair(const float* img, const Grid3& gi, const float* u, const Grid3& g,
+                             float* out_dense, cudaStream_t s);
 // one pyramid step of a float or int16 image: out = (G_1 * in) at even indices;
 // scratch: gout.px * gout.ny * gin.nz floats
 cudaError_t launch_pyramid(int in_type, const void* in, const Grid3& gin, float* scratch,
                            float* out, const Grid3& gout, const Taps& taps, cudaStream_t s);
+// dense device rows into pitched ones, same element type (4 or 2 bytes, aligned)
+bool pitch_rows_supported(const void* dense, int esz);
+cudaError_t launch_pitch_rows(const void* dense, void* pitched, const Grid3& g, int esz,
+                              cudaStream_t s);
 // launch_ic_invert in single precision by way of an interleaved copy of h (scratch:
 // 4 * g.cs floats); two kernels
 bool ic_invert4_supported(const Grid3& g);

@@ -94,3 +94,50 @@ def test_pyramid_and_upsampling(dims, i16):
         w = (pos - lo).reshape([-1 if a == axis else 1 for a in range(4)])
         want = want.take(lo, axis) * (1 - w) + want.take(hi, axis) * w
     assert np.abs(f - want).max() <= 9 * 2.0 ** -24 * np.abs(f).max()
+
+
+@pytest.mark.parametrize("dims", [(1, 5, 4), (2, 2, 2), (33, 9, 13), (40, 1, 9), (64, 31, 6)],
+                         ids=lambda d: "x".join(map(str, d)))
+def test_device_inputs_and_outputs(dims):
+    """Device images, aligned, off by one element, and warped in place, give what
+    host images give; a field read anywhere is the same field."""
+    import torch
+
+    import paper_0909_0928_gb300 as dl
+
+    n = dims[0] * dims[1] * dims[2]
+    shape = dims[::-1]
+
+    def off(a, by=1):  # the same values from a buffer that starts `by` elements in
+        b = torch.empty(n + by, dtype=a.dtype, device="cuda")
+        b[by:] = a.flatten()
+        return b[by:].view(shape)
+
+    for dt, np_t in ((dl.DIR_F32, np.float32), (dl.DIR_I16, np.int16)):
+        S = np.round(400.0 * random_volume(dims, 31)).astype(np_t)
+        M = np.round(400.0 * random_volume(dims, 32)).astype(np_t)
+        got = []
+        for a, b, dev in ((S, M, False), (torch.tensor(S).cuda(), torch.tensor(M).cuda(), True),
+                          (off(torch.tensor(S).cuda()), off(torch.tensor(M).cuda()), True)):
+            p = dl.dir_params_default(levels=1, iters=[5], alpha=0.7)
+            ctx = dl.dir_create(a, b, dims, (1.5, 1.0, 2.0), dt, dev, 0, p)
+            dl.dir_register(ctx)
+            u = dl.dir_get_field(ctx, np.empty((3,) + shape, np.float32))
+            mm = torch.empty(3 * n + 1, device="cuda")
+            dl.dir_get_field(ctx, mm[1:], in_mm=True, out_on_device=True)
+            u64 = dl.dir_get_field_f64(ctx, np.empty((3,) + shape, np.float64))
+            assert np.array_equal(u64, u.astype(np.float64), equal_nan=True)
+            scale = np.array([1.5, 1.0, 2.0], np.float32).reshape(3, 1, 1, 1)
+            assert np.array_equal(mm[1:].cpu().numpy().reshape(u.shape), u * scale, equal_nan=True)
+            img = S.astype(np.float32)
+            w = dl.dir_warp(ctx, img, np.empty(shape, np.float32))
+            d = torch.tensor(img).cuda()
+            for src in (d, off(d), d.clone()):
+                out = src if src is not d else torch.empty_like(d)
+                dl.dir_warp(ctx, src, out, on_device=True)
+                assert np.array_equal(out.cpu().numpy(), w, equal_nan=True)
+            got.append((u, w))
+            dl.dir_destroy(ctx)
+        for u, w in got[1:]:
+            assert np.array_equal(u, got[0][0], equal_nan=True)
+            assert np.array_equal(w, got[0][1], equal_nan=True)
