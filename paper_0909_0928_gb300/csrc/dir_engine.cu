@@ -568,7 +568,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
         if (sched == 4 && n > 0) {
             dirk::LevelGroup G;
             G.taps = c->taps;
-            G.cluster = dirk::level_cluster(&g, 1);
+            G.cluster = dirk::level_cluster(c->variant, &g, 1);
             if (!dirk::level_group_add(G, c->variant, level_args(c, lc, row, cur)))
                 return DIR_EINVAL;
             CK(c, dirk::launch_level(c->variant, c->img_type(l), G, s));
@@ -1384,7 +1384,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
         std::vector<Grid3> held;
         for (int q = 0; q < n; ++q)
             if (level_schedule(ctxs[jobs[q]], l) == 4) held.push_back(ctxs[jobs[q]]->lv[l].g);
-        R.cluster = dirk::level_cluster(held.data(), (int)held.size());
+        R.cluster = dirk::level_cluster(c0->variant, held.data(), (int)held.size());
         for (int q = 0; q < n; ++q) {
             dir_ctx* c = ctxs[jobs[q]];
             if (level_schedule(c, l) != 4) {

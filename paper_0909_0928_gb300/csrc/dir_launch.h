@@ -213,7 +213,7 @@ struct LevelGroup {
     int smem = 0;       // bytes per CTA
 };
 bool level_resident(int variant, const Grid3& g);  // small enough, and its tiles fit
-int level_cluster(const Grid3* g, int n);          // LevelGroup::cluster for these levels
+int level_cluster(int variant, const Grid3* g, int n);  // LevelGroup::cluster for these levels
 bool level_group_add(LevelGroup& G, int variant, const LevelArgs& a);
 cudaError_t launch_level(int variant, int img_type, const LevelGroup& G, cudaStream_t s);
 

@@ -517,45 +517,55 @@ bool level_tiles(const Grid3& g, int variant, int C, int* tr, int* tp, int* smem
 }
 
 template <int V, typename TI>
-cudaError_t setup_level(int* clusters = nullptr) {
-    // KernelSetup's per_sm keeps how many clusters of kLevelCluster CTAs the
-    // device can hold (0: none, e.g. a partitioned GPU)
+cudaError_t setup_level() {
     static KernelSetup setup;  // per instantiation
-    cudaError_t e = setup_kernel(setup, level_kernel<V, TI>, kLevelMaxSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(level_kernel<V, TI>,
-                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess || !clusters) return e;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kLevelCluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(kLevelCluster);
-    cfg.blockDim = dim3(LNT);
-    cfg.dynamicSmemBytes = kLevelMaxSmem;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(clusters, level_kernel<V, TI>, &cfg);
+    const cudaError_t e = setup_kernel(setup, level_kernel<V, TI>, kLevelMaxSmem);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(
+                                  level_kernel<V, TI>,
+                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
-// Whether the current device can hold a cluster of the kernel (asked once)
-bool clusters_available() {
+// How many clusters of 1 .. kLevelCluster CTAs the current device runs at once
+// (one CTA per SM; a cluster stays within a GPC), asked once per device; nullptr
+// where it holds none of kLevelCluster / 2 CTAs (e.g. a partitioned GPU).
+struct ActiveClusters {
+    int n[kLevelCluster + 1];
+};
+const ActiveClusters* active_clusters() {
     static std::atomic<int> known[KernelSetup::kMaxDevices];  // 0 unknown, 1 no, 2 yes
+    static ActiveClusters table[KernelSetup::kMaxDevices];
+    static std::mutex mutex;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= KernelSetup::kMaxDevices)
-        return false;
+        return nullptr;
     int k = known[dev].load(std::memory_order_acquire);
     if (k == 0) {
-        int n = 0;
-        if (setup_level<0, float>(&n) != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
+        std::lock_guard<std::mutex> lock(mutex);
+        ActiveClusters& t = table[dev];
+        const bool ok = setup_level<0, float>() == cudaSuccess;
+        for (int C = 1; C <= kLevelCluster; ++C) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)C;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3((unsigned)C);
+            cfg.blockDim = dim3(LNT);
+            cfg.dynamicSmemBytes = kLevelMaxSmem;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (!ok ||
+                cudaOccupancyMaxActiveClusters(&n, level_kernel<0, float>, &cfg) != cudaSuccess)
+                n = 0;
+            t.n[C] = n;
         }
-        k = n > 0 ? 2 : 1;
+        cudaGetLastError();
+        k = t.n[kLevelCluster / 2] > 0 ? 2 : 1;
         known[dev].store(k, std::memory_order_release);
     }
-    return k == 2;
+    return k == 2 ? &table[dev] : nullptr;
 }
 
 template <int V, typename TI>
@@ -591,21 +601,45 @@ cudaError_t launch_level_types(int variant, const LevelGroup& G, int smem, cudaS
 
 }  // namespace
 
-// CTAs per cluster for a launch over n levels: one per 128 voxels of the largest
-// (16x16x8: 2.8 us per passive iteration with 16 CTAs, 2.9 with 8, 3.3 with 4),
-// as many as lets all the clusters run at once (a cluster of 16 takes a GPC).
-int level_cluster(const Grid3* g, int n) {
-    const int most = n <= 8 ? kLevelCluster : kLevelCluster / 2;
-    int c = 1;
-    for (int j = 0; j < n; ++j)
-        while (c < most && 128LL * c < (long long)g[j].nx * g[j].ny * g[j].nz) c *= 2;
-    return c;
+// CTAs per cluster for a launch over n levels.  An iteration takes about 1.6 us +
+// 0.04 us per CTA (barriers) + 0.002 us per voxel of the largest tile (Eq. 1,
+// measured / this: 16x16x8 16 CTAs 2.66 / 2.5, 8: 2.48 / 2.4, 6: 2.76 / 2.7, 5: 3.0;
+// 32x32x16 16: 3.83 / 4.3, 8: 5.9 / 6.0, 6: 7.7 / 7.3), and clusters that do not
+// run at once take turns.  A GB300 holds 7 clusters of 16 CTAs, 15 of 8, 23 of 6:
+// 16 levels of 32x32x16 took 11.8 us an iteration in two turns of 8 CTAs and
+// take 7.8 in one of 6 (the grouped split kernels: 10.4); 8 levels of 16x16x8
+// 5.3 us in two turns of 16, now 2.5 in one of 8.
+int level_cluster(int variant, const Grid3* g, int n) {
+    const ActiveClusters* active = active_clusters();
+    int best_c = kLevelCluster / 2;
+    double best = 1e30;
+    for (int C = 1; active && C <= kLevelCluster; ++C) {
+        if (active->n[C] < 1) continue;
+        int tile = 0;
+        for (int j = 0; j < n && tile >= 0; ++j) {
+            if (j > 0 && g[j].nx == g[j - 1].nx && g[j].ny == g[j - 1].ny && g[j].nz == g[j - 1].nz)
+                continue;
+            int tr, tp, smem;
+            if (level_tiles(g[j], variant, C, &tr, &tp, &smem))
+                tile = std::max(tile, tr * tp * g[j].nx);
+            else
+                tile = -1;  // does not fit
+        }
+        if (tile < 0) continue;
+        const int turns = (n + active->n[C] - 1) / active->n[C];
+        const double us = turns * (1.6 + 0.04 * C + 0.002 * tile);
+        if (us < best) {
+            best = us;
+            best_c = C;
+        }
+    }
+    return best_c;
 }
 
 bool level_resident(int variant, const Grid3& g) {
     int tr, tp, smem;
     return (long long)g.nx * g.ny * g.nz <= kLevelMaxVoxels &&
-           level_tiles(g, variant, kLevelCluster / 2, &tr, &tp, &smem) && clusters_available();
+           level_tiles(g, variant, kLevelCluster / 2, &tr, &tp, &smem) && active_clusters();
 }
 
 bool level_group_add(LevelGroup& G, int variant, const LevelArgs& a) {
