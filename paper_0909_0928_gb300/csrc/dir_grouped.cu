@@ -22,13 +22,15 @@ static_assert(sizeof(XYGroup) < 30000 && sizeof(ZSGroup) < 30000 && sizeof(ZDGro
               "grouped launch parameters must fit the kernel parameter space");
 
 __device__ __forceinline__ int group_job(const int* first, int n, int b) {
-    int j = 0;
-    while (j + 1 < n && b >= first[j + 1]) ++j;
+    int j = 0;  // independent compares, not a walk (first[k] ascends up to k = n)
+#pragma unroll
+    for (int k = 1; k < kGroupMax; ++k) j += (k < n && b >= first[k]) ? 1 : 0;
     return j;
 }
 
 __device__ __forceinline__ BlockPos group_pos(int lb, int gx, int gy, int gz) {
-    return {lb % gx, (lb / gx) % gy, lb / (gx * gy), gx, gy, gz};
+    const unsigned row = (unsigned)lb / (unsigned)gx, z = row / (unsigned)gy;
+    return {lb - (int)row * gx, (int)(row - z * gy), (int)z, gx, gy, gz};
 }
 
 __global__ void __launch_bounds__(8 * S2Y)
