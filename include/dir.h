@@ -121,12 +121,12 @@ typedef struct {
                                     2 (default): as 4 where it applies, and on levels of at most
                                     16,384 voxels without a stop test or timing all iterations
                                     in one launch, the field in the shared memory of a
-                                    thread-block cluster.  dir_register_noalloc
-                                    has no scratch for the form of 4: there 2 is split for Eqs.
-                                    (1)-(2) on every level and for Eqs. (3)-(6) on levels of at
-                                    most 2^21 voxels, else fused on the small levels that one
-                                    block per SM covers in two-plane chunks (e.g. 64 x 64 x 25),
-                                    else 0, and 4 is 3 */
+                                    thread-block cluster.  Where the scratch of
+                                    dir_register_noalloc has no room for the form of 4: there 2
+                                    is split for Eqs. (1)-(2) on every level and for Eqs. (3)-(6)
+                                    on levels of at most 2^21 voxels, else fused on the small
+                                    levels that one block per SM covers in two-plane chunks
+                                    (e.g. 64 x 64 x 25), else 0, and 4 is 3 */
     int plain_kernels;           /* 0 (default): the production kernels (TMA-fed bricks and
                                     plane rings, packed smoothing, fused small levels).  1: the
                                     plain-load kernels with the same per-voxel arithmetic and

@@ -315,8 +315,8 @@ static bool level_split_ok(const dir_ctx* c, int l) {
 // against 169.7 and 148.6 on the finest level, 21.7 against 27.8 on
 // 128x128x50, 10.2 against 10.5 on 64x64x25; Eq. 6: 170.8 against 229.1 and
 // 207.8, 36.6 against 45.4, 16.8 against 17.8.  It needs the D scratch
-// (dir_ctx::C), allocated for the levels that run it; without one
-// (dir_register_noalloc) a level runs what the rules below give.
+// (dir_ctx::C), allocated for the levels that run it; where dir_register_noalloc
+// has no room for it a level runs what the rules below give.
 static bool level_wants_d(const dir_ctx* c, int l) {
     if (c->variant < 2 || !level_split_ok(c, l)) return false;
     return c->p.fuse == 2 || c->p.fuse == 4;
@@ -328,9 +328,16 @@ static bool level_wants_d(const dir_ctx* c, int l) {
 // kernel gains from 8 (38.3 us against 42.3 us)
 constexpr int kZdMaxDepth = 4;
 
-static size_t level_d_bytes(const dir_ctx* c, int l) {
-    return (size_t)dirk::force_d_planes(c->variant, c->lv[l].g) * (size_t)c->lv[l].g.cs *
+static size_t level_d_bytes(const dir_ctx* c, int l, bool writes_u) {
+    return (size_t)dirk::force_d_planes(c->variant, writes_u) * (size_t)c->lv[l].g.cs *
            sizeof(float);
+}
+static size_t level_d_bytes(const dir_ctx* c, int l) {  // in its preferred form
+    return level_d_bytes(c, l, dirk::force_d_writes_u(c->lv[l].g));
+}
+// the preferred form where the scratch holds it, else u formed again
+static bool level_writes_u(const dir_ctx* c, int l) {
+    return dirk::force_d_writes_u(c->lv[l].g) && c->C_bytes >= level_d_bytes(c, l, true);
 }
 
 // The interleaved mid-space field of Eq. 6's output step, in the scratch too
@@ -382,7 +389,7 @@ static int level_schedule(const dir_ctx* c, int l) {
     const Grid3& g = c->lv[l].g;
     const bool split_ok = level_split_ok(c, l);
     if (level_wants_resident(c, l) && dirk::level_resident(c->variant, g)) return 4;
-    if (level_wants_d(c, l) && c->C && c->C_bytes >= level_d_bytes(c, l)) return 3;
+    if (level_wants_d(c, l) && c->C && c->C_bytes >= level_d_bytes(c, l, false)) return 3;
     const bool eqs12 = c->variant == 0 || c->variant == 1;
     const bool fused_ok = c->p.stop_mode == 0 && dirk::fused_supported(c->variant) &&
                           c->field_type == c->real_type && c->img_type(l) == c->real_type;
@@ -672,7 +679,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                         dirk::ForceArgs za = fa, ta = fa;
                         za.depth = std::min(zs_depth, kZdMaxDepth);
                         za.u = ta.u = tbuf;
-                        d_scratch(c, g, dirk::force_d_writes_u(g), za, ta);
+                        d_scratch(c, g, level_writes_u(c, l), za, ta);
                         CK(c, dirk::launch_force_d(c->variant, za, ta, c->taps, s));
                         c->launches += 3;
                     } else {
@@ -1716,7 +1723,7 @@ extern "C" int dir_autotune(dir_ctx* c, int reps, int* shapes_out) {
         // schedule 3: the z + D and stencil force kernels, D in the scratch
         dirk::ForceArgs za = fa, ta = fa;
         if (sched == 3) {
-            d_scratch(c, g, dirk::force_d_writes_u(g), za, ta);
+            d_scratch(c, g, level_writes_u(c, l), za, ta);
         }
         for (int di = 0; di < (sched == 2 ? 5 : 4) && rc == DIR_OK; ++di) {
             const int d = depths[di];
@@ -1884,6 +1891,17 @@ extern "C" int dir_register_noalloc(const float* static_img, const float* moving
         return DIR_EINVAL;
     }
 
+    // what is left holds the D scratch of Eqs. 3-6 and Eq. 6's interleaved field,
+    // as far as they fit (128x128x64, active, 200/100/50: 3.94 ms without, now 3.53)
+    const size_t offC = at;
+    for (int l = 0; l < c.levels; ++l)
+        if (p.iters[c.levels - 1 - l] > 0 && level_wants_d(&c, l))
+            c.C_bytes = std::max(c.C_bytes, level_d_bytes(&c, l));
+    if (c.variant == DIR_INVERSE_CONSISTENT && level_wants_d(&c, 0) &&
+        dirk::ic_invert4_supported(c.lv[0].g))
+        c.C_bytes = std::max(c.C_bytes, ic_bytes(&c));
+    c.C_bytes = std::min(c.C_bytes, kNoallocScratchBytes - offC);
+
     // device address of the static scratch, once per device, that device current
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1917,6 +1935,7 @@ extern "C" int dir_register_noalloc(const float* static_img, const float* moving
     }
     c.A = base + offA;
     c.B = base + offB;
+    c.C = c.C_bytes > 0 ? base + offC : nullptr;
     c.red = reinterpret_cast<double*>(base + offRed);
     c.corr = want_corr ? reinterpret_cast<double*>(base + offCorr) : nullptr;
     c.lhist = reinterpret_cast<double*>(base + offL);

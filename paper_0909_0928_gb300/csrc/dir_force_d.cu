@@ -82,7 +82,7 @@ cudaError_t launch_st(const ForceArgs& a, const Taps& taps, cudaStream_t s) {
 template <int V, typename TI>
 cudaError_t launch_d_pair(const ForceArgs& zd, const ForceArgs& st, const Taps& taps,
                           cudaStream_t s) {
-    if (!force_d_writes_u(zd.g)) {  // large levels: bricks of 4 (z + D), 4 or 8 planes
+    if (st.u != zd.v) {  // u formed again: bricks of 4 (z + D), 4 or 8 planes
         const cudaError_t e = launch_zd<V, 4, TI, false>(zd, taps, s);
         if (e != cudaSuccess) return e;
         return st.depth >= 8 ? launch_st<V, 8, TI, false>(st, taps, s)
@@ -135,9 +135,7 @@ bool force_d_supported(int variant, const ForceArgs& a, const Taps& taps) {
 // 256x256x100 103.2 -> 96.1 / 117.1 -> 114.1.
 bool force_d_writes_u(long long voxels) { return voxels <= (1LL << 20); }
 
-int force_d_planes(int variant, const Grid3& g) {
-    return (variant == 5 ? 2 : 1) + (force_d_writes_u(g) ? 3 : 0);
-}
+int force_d_planes(int variant, bool writes_u) { return (variant == 5 ? 2 : 1) + (writes_u ? 3 : 0); }
 
 // Brick depth of the force pass (the z + D pass caps it at 4): 8 for Eqs. 3-5
 // where such bricks number three per SM, else 4 where those number one per SM,

@@ -101,15 +101,16 @@ cudaError_t launch_force_zs(int variant, const ForceArgs& a, const Taps& taps, c
 // voxel (dir_split_d.cuh): after launch_smooth_xy, the z + D pass (zd: u = t,
 // dbuf / dbuf2 = the D it writes) and the stencil force pass (st: u = t, v = the
 // field out, dbuf / dbuf2 = that D), each with its own brick depth (1, 2, 4 or
-// 8; 6 runs as 4).  On levels where force_d_writes_u, zd.v and st.u are u, which
-// the first writes and the second reads.  force_d_planes: floats per voxel of
-// the scratch for D (1, Eq. 6: 2) and, there, u (3).
+// 8; 6 runs as 4).  Where zd.v and st.u are the same array, it is u, which the
+// first writes and the second reads (preferred where force_d_writes_u); else both
+// form u from t.  force_d_planes: floats per voxel of the scratch for D (1, Eq. 6:
+// 2) and, if written, u (3).
 bool force_d_supported(int variant, const ForceArgs& a, const Taps& taps);
 bool force_d_writes_u(long long voxels);
 inline bool force_d_writes_u(const Grid3& g) {
     return force_d_writes_u((long long)g.nx * g.ny * g.nz);
 }
-int force_d_planes(int variant, const Grid3& g);
+int force_d_planes(int variant, bool writes_u);
 int force_d_depth(int variant, const Grid3& g, int num_sms);
 cudaError_t launch_force_d(int variant, const ForceArgs& zd, const ForceArgs& st, const Taps& taps,
                            cudaStream_t s);

@@ -141,3 +141,25 @@ def test_device_inputs_and_outputs(dims):
         for u, w in got[1:]:
             assert np.array_equal(u, got[0][0], equal_nan=True)
             assert np.array_equal(w, got[0][1], equal_nan=True)
+
+
+@pytest.mark.parametrize("nz", [60, 64, 90], ids=["D and u fit", "D fits", "neither fits"])
+@pytest.mark.parametrize("variant", [2, 5], ids=["active", "inverse_consistent"])
+def test_noalloc_scratch_forms(variant, nz):
+    """128 x 128 x nz in 48 MiB: every form of the iteration gives the field of a
+    context, whose scratch is its own."""
+    import torch
+
+    import paper_0909_0928_gb300 as dl
+
+    dims = (128, 128, nz)
+    S, M = (torch.tensor(np.round(400.0 * random_volume(dims, k)).astype(np.float32)).cuda()
+            for k in (41, 42))
+    p = dl.dir_params_default(levels=1, iters=[3], alpha=0.7)
+    out = torch.empty((3,) + dims[::-1], device="cuda")
+    dl.dir_register_noalloc(S, M, dims, variant, p, out)
+    ctx = dl.dir_create(S, M, dims, (1.0, 1.0, 1.0), dl.DIR_F32, True, variant, p)
+    dl.dir_register(ctx)
+    want = dl.dir_get_field(ctx, np.empty(out.shape, np.float32))
+    dl.dir_destroy(ctx)
+    assert np.array_equal(out.cpu().numpy(), want, equal_nan=True)
