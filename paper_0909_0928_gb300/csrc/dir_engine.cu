@@ -512,6 +512,23 @@ static dirk::ForceArgs level_force_args(const dir_ctx* c, int lc) {
     return fa;
 }
 
+// The stop test after iteration `it` of level lc, whose sums are `row`
+static dirk::StopTest level_stop_test(const dir_ctx* c, int lc, int row, int it) {
+    const Grid3& g = c->lv[c->levels - 1 - lc].g;
+    dirk::StopTest q;
+    q.red = c->red;
+    q.corr = c->p.stop_mode == 2 ? c->corr : nullptr;
+    q.n = (double)g.nx * g.ny * g.nz;
+    q.lhist = c->lhist;
+    q.t = row;
+    q.level_first = c->level_first[lc];
+    q.window = c->p.stop_window;
+    q.eps = c->p.eps;
+    q.stop_iter = c->ctl + lc;
+    q.iter = it;
+    return q;
+}
+
 static dirk::SmoothArgs level_smooth_args(const dir_ctx* c, int lc) {
     const int l = c->levels - 1 - lc;
     dirk::SmoothArgs sa;
@@ -655,6 +672,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                                               : dirk::force_zs_depth(c->variant, g, c->num_sms);
             const int first_depth = dirk::force_brick_depth(g, c->num_sms);
             const bool pdl = level_pdl(c, g, timed);
+            dirk::StopTest test;  // of the iteration before
             for (int it = 0; it < n; ++it, ++row) {
                 cudaEvent_t* e = timed ? &c->tev[3 * (size_t)c->n_timed] : nullptr;
                 if (timed && record(c, e[0], s, capturing) != DIR_OK) return DIR_ECUDA;
@@ -671,7 +689,8 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                 } else {
                     xa.iter = it;
                     xa.pdl = pdl;
-                    CK(c, dirk::launch_smooth_xy(xa, c->num_sms, s));
+                    if (test.red) xa.stop_iter = nullptr;
+                    CK(c, dirk::launch_smooth_xy(xa, c->num_sms, s, test));
                     if (timed && record(c, e[1], s, capturing) != DIR_OK) return DIR_ECUDA;
                     fa.depth = zs_depth;
                     fa.pdl = pdl;
@@ -690,11 +709,12 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
                 }
                 if (timed && record(c, e[2], s, capturing) != DIR_OK) return DIR_ECUDA;
                 if (c->p.stop_mode >= 1) {
-                    CK(c, dirk::launch_stop_test(c->red, c->p.stop_mode == 2 ? c->corr : nullptr,
-                                                 (double)g.nx * g.ny * g.nz, c->lhist, row,
-                                                 c->level_first[lc], c->p.stop_window, c->p.eps,
-                                                 c->ctl + lc, it, s));
-                    c->launches += 1;
+                    // the next iteration's x/y kernel makes the test; the last's here
+                    test = level_stop_test(c, lc, row, it);
+                    if (it == n - 1) {
+                        CK(c, dirk::launch_stop_test(test, s));
+                        c->launches += 1;
+                    }
                 }
                 if (timed) c->n_timed += 1;
             }
@@ -722,10 +742,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
             c->launches += 1;
             if (c->p.stop_mode >= 1) {
                 // Sec. 2.4 on the relative norm, or (stop_mode 2) on the correlation
-                CK(c, dirk::launch_stop_test(c->red, c->p.stop_mode == 2 ? c->corr : nullptr,
-                                             (double)g.nx * g.ny * g.nz, c->lhist, row,
-                                             c->level_first[lc], c->p.stop_window, c->p.eps,
-                                             c->ctl + lc, it, s));
+                CK(c, dirk::launch_stop_test(level_stop_test(c, lc, row, it), s));
                 c->launches += 1;
             }
             if (timed && record(c, e[1], s, capturing) != DIR_OK) return DIR_ECUDA;

@@ -67,6 +67,21 @@ struct SmoothArgs {
                          // boxes per strip; 0 = the launcher's rule)
     bool pdl = false;    // as ForceArgs::pdl (the x/y kernel)
 };
+// Stop test of Sec. 2.4 after iteration `iter` of a level, whose sums are row t, on
+// the relative norm (corr == nullptr) or on the correlation coefficient of the
+// warped image with its reference (corr: the four sums of each iteration, n: voxels
+// of the level): lhist[t] is written, and *stop_iter = iter where it holds.
+struct StopTest {
+    const double* red = nullptr;  // null: no test
+    const double* corr = nullptr;
+    double n = 0.0;
+    double* lhist = nullptr;
+    int t = 0, level_first = 0, window = 0;
+    double eps = 0.0;
+    int* stop_iter = nullptr;
+    int iter = 0;
+};
+
 // plain = true: the 32 x 8 tile kernel (smooth_kernel) for every storage type
 // instead of the packed single-precision kernels
 cudaError_t launch_smooth(bool fp64, const SmoothArgs& a, int num_sms, cudaStream_t s,
@@ -76,7 +91,10 @@ cudaError_t launch_smooth(bool fp64, const SmoothArgs& a, int num_sms, cudaStrea
 // three components, radius 3): out = G_y * G_x * in.  With
 // launch_force_zs, which applies G_z, one smoothing + force iteration.
 bool smooth_xy_supported(const SmoothArgs& a);
-cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s);
+// test: the stop test of the iteration before, made by every block first (a.stop_iter
+// is then not read)
+cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s,
+                             const StopTest& test = StopTest());
 
 // Force pass of Eqs. 1-2 whose u is G_z * t, t = a.u the output of
 // launch_smooth_xy (single-precision field, float or int16 images, radius 3):
@@ -279,12 +297,7 @@ cudaError_t launch_import(bool fp64, int out_type, const float* dense, void* pit
 // one bounded wait on an mbarrier that never completes; sets kErrTmaTimeout
 // in *err when it gives up after limit_ns
 cudaError_t launch_wait_probe(int* err, unsigned long long limit_ns, cudaStream_t s);
-// stop test of Sec. 2.4 for iteration t of a level on the relative norm
-// (corr == nullptr) or on the correlation coefficient of the warped image with
-// its reference (corr: the four sums of each iteration, n: voxels of the level)
-cudaError_t launch_stop_test(const double* red, const double* corr, double n, double* lhist,
-                             int t, int level_first, int window, double eps, int* stop_iter,
-                             int iter_in_level, cudaStream_t s);
+cudaError_t launch_stop_test(const StopTest& q, cudaStream_t s);  // one thread
 // correlation coefficient from Sum d^2 and the four sums of CorrSums over n voxels
 __host__ __device__ inline double correlation_from_sums(double sdd, const double* c, double n) {
     const double sb = c[0], sbb = c[1], sd = c[2], sbd = c[3];

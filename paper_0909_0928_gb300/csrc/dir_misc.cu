@@ -10,6 +10,7 @@
 #include "dir_common.cuh"
 #include "dir_launch.h"
 #include "dir_pair.cuh"
+#include "dir_stop.cuh"
 
 namespace dirk {
 
@@ -352,21 +353,7 @@ __global__ void pyramid_z_kernel(const float* __restrict__ t, int nz, float* __r
     out[offs(go, X, Y, Z)] = acc;
 }
 
-// Sec. 2.4: l(t) = sum|du| / sum|u|; stop the level after iteration t when
-// |l(t) - l(t - window)| <= eps (both defined).  One thread.
-__global__ void stop_test_kernel(const double* __restrict__ red, const double* __restrict__ corr,
-                                 double n, double* lhist, int t, int level_first, int window,
-                                 double eps, int* stop_iter, int iter_in_level) {
-    if (*stop_iter < iter_in_level) return;
-    const double B = red[3 * t + 2];
-    const double l = corr ? correlation_from_sums(red[3 * t], corr + 4 * t, n)
-                          : (B > 0.0 ? red[3 * t + 1] / B : nan(""));
-    lhist[t] = l;
-    if (iter_in_level >= window && t - window >= level_first) {
-        const double lp = lhist[t - window];
-        if (!isnan(l) && !isnan(lp) && fabs(l - lp) <= eps) *stop_iter = iter_in_level;
-    }
-}
+__global__ void stop_test_kernel(const StopTest q) { stop_test(q, true); }
 
 // Dispatch on (arithmetic, field storage): double/double, float/float,
 // float/bf16.  `CALL` sees the types as Real and TF.
@@ -536,11 +523,9 @@ cudaError_t launch_wait_probe(int* err, unsigned long long limit_ns, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_stop_test(const double* red, const double* corr, double n, double* lhist,
-                             int t, int level_first, int window, double eps, int* stop_iter,
-                             int iter_in_level, cudaStream_t s) {
-    stop_test_kernel<<<1, 1, 0, s>>>(red, corr, n, lhist, t, level_first, window, eps, stop_iter,
-                                     iter_in_level);
+cudaError_t launch_stop_test(const StopTest& q, cudaStream_t s) {
+    if (q.red == nullptr) return cudaErrorInvalidValue;
+    stop_test_kernel<<<1, 1, 0, s>>>(q);
     return cudaGetLastError();
 }
 

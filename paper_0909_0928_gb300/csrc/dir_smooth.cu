@@ -22,6 +22,7 @@
 #include "dir_smooth2.cuh"
 #include "dir_split.cuh"
 #include "dir_stencil.cuh"
+#include "dir_stop.cuh"
 #include "dir_xy.cuh"
 
 namespace dirk {
@@ -189,15 +190,23 @@ __global__ void __launch_bounds__(8 * TY, 16 / TY * 8)
 // smooth2_kernel, in two forms: warps marching down y (dir_xy.cuh) on levels
 // that fill the GPU with them, and on smaller ones blocks of 32 x 16 tiles
 // (sxy_block), whose shorter chain of dependent steps counts there.
+// With a stop test every block makes it for itself before it starts (0.3 us on
+// the loads of the sums, which the flag alone would cost too), instead of a launch
+// of its own between two iterations (1.7 us and the gap to the next kernel).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(32 * XYWARPS)
     smooth_xy_strip_kernel(const __grid_constant__ CUtensorMap tmap, const SmoothArgs a,
-                           const XYStrips st) {
+                           const XYStrips st, const StopTest test) {
+    if (test.red != nullptr && block_stop_test(test, blockIdx.x == 0)) return;
     xy_strip_block(&tmap, a, st, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(8 * S2Y)
-    smooth_xy_kernel(const __grid_constant__ CUtensorMap tmap, const SmoothArgs a, int zchunk) {
+    smooth_xy_kernel(const __grid_constant__ CUtensorMap tmap, const SmoothArgs a, int zchunk,
+                     const StopTest test) {
+    if (test.red != nullptr &&
+        block_stop_test(test, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0))
+        return;
     sxy_block<XYR, S2Y>(&tmap, a, zchunk, BlockPos::of_grid());
 }
 
@@ -403,7 +412,8 @@ static cudaError_t launch_s2t(const SmoothArgs& a, int num_sms, cudaStream_t s) 
     return launch_s2<R, S2Y>(a, num_sms, s);
 }
 
-static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, cudaStream_t s) {
+static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, const StopTest& test,
+                              cudaStream_t s) {
     using G = SXYSmem<XYR, S2Y>;
     CUtensorMap map;
     if (!make_s2_map<XYR, S2Y>(&map, a.in, a.g, a.ncomp)) return cudaErrorInvalidValue;
@@ -428,10 +438,12 @@ static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, cudaStream_t s) 
     if (zc > a.g.nz) zc = a.g.nz;
     const int chunks = (a.g.nz + zc - 1) / zc;
     const dim3 grid((a.g.nx + S2X - 1) / S2X, (a.g.ny + S2Y - 1) / S2Y, chunks * a.ncomp);
-    return launch_ex(smooth_xy_kernel, grid, dim3(8 * S2Y, 1, 1), G::SMEM, s, a.pdl, map, a, zc);
+    return launch_ex(smooth_xy_kernel, grid, dim3(8 * S2Y, 1, 1), G::SMEM, s, a.pdl, map, a, zc,
+                     test);
 }
 
-static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, cudaStream_t s) {
+static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, const StopTest& test,
+                                    cudaStream_t s) {
     CUtensorMap map;
     if (!make_xy_strip_map(&map, a.in, a.g)) return cudaErrorInvalidValue;
     static KernelSetup setup;
@@ -443,7 +455,7 @@ static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, cudaStream
                                 : xy_strip_boxes(&a.g, 1, per_sm * num_sms * XYWARPS);
     const XYStrips st = xy_strips(a.g, nb);
     return launch_ex(smooth_xy_strip_kernel, dim3((unsigned)st.blocks()), dim3(32 * XYWARPS, 1, 1),
-                     XYSMEM, s, a.pdl, map, a, st);
+                     XYSMEM, s, a.pdl, map, a, st, test);
 }
 
 template <typename Real, int R, typename TIN, typename TOUT>
@@ -483,10 +495,11 @@ bool smooth_xy_supported(const SmoothArgs& a) {
     return a.ncomp == 3 && a.in_type == kStoreF32 && a.out_type == kStoreF32 && a.taps.R == XYR;
 }
 
-cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s,
+                             const StopTest& test) {
     if (!smooth_xy_supported(a)) return cudaErrorInvalidValue;
-    return xy_use_strips(&a.g, 1, num_sms) ? launch_xy_strips(a, num_sms, s)
-                                           : launch_sxy(a, num_sms, s);
+    return xy_use_strips(&a.g, 1, num_sms) ? launch_xy_strips(a, num_sms, test, s)
+                                           : launch_sxy(a, num_sms, test, s);
 }
 
 cudaError_t launch_smooth(bool fp64, const SmoothArgs& a, int num_sms, cudaStream_t s,

@@ -163,3 +163,38 @@ def test_noalloc_scratch_forms(variant, nz):
     want = dl.dir_get_field(ctx, np.empty(out.shape, np.float32))
     dl.dir_destroy(ctx)
     assert np.array_equal(out.cpu().numpy(), want, equal_nan=True)
+
+
+@pytest.mark.parametrize("dims", [(31, 33, 7), (129, 128, 60)], ids=["tiles", "strips"])
+@pytest.mark.parametrize("mode", [1, 2], ids=["norm", "correlation"])
+def test_stop_test_in_the_smoothing_kernel(dims, mode):
+    """The stop test made by the next x/y kernel ends a level where the test's own
+    kernel does (plain kernels), with the same field.  eps lies half way between
+    two values of |l(t) - l(t - window)| of a run that does not stop, far from the
+    rounding of the sums."""
+    import paper_0909_0928_gb300 as dl
+
+    S = np.round(400.0 * random_volume(dims, 51)).astype(np.float32)
+    M = np.round(400.0 * random_volume(dims, 52)).astype(np.float32)
+
+    def run(n, **kw):
+        p = dl.dir_params_default(levels=1, iters=[n], alpha=0.7, **kw)
+        ctx = dl.dir_create(S, M, dims, (1.0, 1.0, 1.0), dl.DIR_F32, False, 0, p)
+        try:
+            st = dl.dir_register(ctx)
+            u = dl.dir_get_field(ctx, np.empty((3,) + dims[::-1], np.float32))
+            l = (dl.dir_get_history if mode == 1 else dl.dir_get_correlation)(ctx, n)
+            return st.iters_run[0], u, l
+        finally:
+            dl.dir_destroy(ctx)
+
+    n, w = 12, 2
+    l = run(n, correlation=1)[2]
+    l = l[1:]  # no |u| before the first update
+    l = l[:, 1] / l[:, 2] if mode == 1 else l
+    step = np.sort(np.abs(l[w:] - l[:-w]))
+    eps = float(step[4] + step[5]) / 2
+    kw = dict(stop_mode=mode, eps=eps, stop_window=w)
+    a, b = run(n, **kw), run(n, plain_kernels=1, **kw)
+    assert a[0] == b[0] and w < a[0] < n
+    assert np.array_equal(a[1], b[1], equal_nan=True)
