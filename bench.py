@@ -108,14 +108,19 @@ KERNEL_SOURCES = {
                       "dir_force_law.cuh", "dir_common.cuh"],
     "fused_small_kernel": ["dir_fused.cu", "dir_smooth2.cuh", "dir_force_kernel.cuh",
                            "dir_force_law.cuh", "dir_common.cuh"],
-    "smooth_xy_kernel": ["dir_smooth.cu", "dir_split.cuh", "dir_smooth2.cuh", "dir_common.cuh"],
-    "force_zs_kernel": ["dir_force_zs.cu", "dir_split.cuh", "dir_force_gm.cuh",
+    "smooth_xy_strip_kernel": ["dir_smooth.cu", "dir_xy.cuh", "dir_pair.cuh", "dir_stop.cuh",
+                               "dir_stencil.cuh", "dir_common.cuh"],
+    "smooth_xy_kernel": ["dir_smooth.cu", "dir_split.cuh", "dir_smooth2.cuh", "dir_pair.cuh",
+                         "dir_stop.cuh", "dir_common.cuh"],
+    "force_zs_kernel": ["dir_force_zs.cu", "dir_split.cuh", "dir_pair.cuh", "dir_force_gm.cuh",
                         "dir_force_kernel.cuh", "dir_force_law.cuh", "dir_stencil.cuh",
                         "dir_common.cuh"],
-    "force_zd_kernel": ["dir_force_d.cu", "dir_split_d.cuh", "dir_split.cuh",
+    "force_zd_kernel": ["dir_force_d.cu", "dir_split_d.cuh", "dir_split.cuh", "dir_pair.cuh",
                         "dir_force_kernel.cuh", "dir_stencil.cuh", "dir_common.cuh"],
-    "force_st_kernel": ["dir_force_d.cu", "dir_split_d.cuh", "dir_force_kernel.cuh",
-                        "dir_force_law.cuh", "dir_stencil.cuh", "dir_common.cuh"],
+    "force_st_kernel": ["dir_force_d.cu", "dir_split_d.cuh", "dir_pair.cuh",
+                        "dir_force_kernel.cuh", "dir_force_law.cuh", "dir_stencil.cuh",
+                        "dir_common.cuh"],
+    "level_kernel": ["dir_level.cu", "dir_pair.cuh", "dir_stencil.cuh", "dir_common.cuh"],
 }
 
 
@@ -821,11 +826,12 @@ def main():
     kernel_of = {"force": "force_tma_kernel" if args.variant_id in (0, 1) else "force_tma_gm_kernel",
                  "fused": "fused2_kernel", "smooth": "smooth2_kernel"}
     if schedule == 2:  # split Gaussian: x/y kernel, then z pass + force (same bytes per voxel)
-        kernel_of.update(force="force_zs_kernel", smooth="smooth_xy_kernel")
+        kernel_of.update(force="force_zs_kernel", smooth="smooth_xy_strip_kernel")
     if schedule == 3:  # Eqs. 3-6: x/y kernel, z + D kernel, stencil force kernel
-        kernel_of.update(force="force_zd_kernel+force_st_kernel", smooth="smooth_xy_kernel")
-        # z + D: t 12, S 4, M 4, u 12, D 4 (Eq. 6: + d 4); force: D 4, S 4, u 12, v 12 (+ d 4)
-        bytes_pv["force"] = 68 if args.variant_id != 5 else 76
+        kernel_of.update(force="force_zd_kernel+force_st_kernel", smooth="smooth_xy_strip_kernel")
+        # z + D: t 12, S 4, M 4, D 4 (Eq. 6: + d 4); force: D 4, S 4, t 12, v 12 (+ d 4); u is
+        # formed from t in both on a level of this size
+        bytes_pv["force"] = 56 if args.variant_id != 5 else 64
     per_kernel = {}
     for k, (ms, n) in kt.items():
         if n:
@@ -882,10 +888,10 @@ def main():
             per_variant[name] = {"ms_p50": med, "voxel_updates_per_s": vu_step / (med / 1e3)}
         # the finest-level iteration of Eqs. 3 and 6 in the default schedule
         # (x/y kernel, z + D kernel, stencil force kernel), untimed as above.
-        # Algorithmic bytes per voxel: x/y 24, z + D 36 (t 12, S 4, M 4, u 12,
-        # D 4; Eq. 6 + d 4), force 32 (D 4, S 4, u 12, v 12; Eq. 6 + d 4)
+        # Algorithmic bytes per voxel: x/y 24, z + D 24 (t 12, S 4, M 4, D 4;
+        # Eq. 6 + d 4), force 32 (D 4, S 4, t 12, v 12; Eq. 6 + d 4)
         try:
-            for vid, bpv in ((2, 92), (5, 100)):
+            for vid, bpv in ((2, 80), (5, 88)):
                 it_ms = (untimed_ms(fine_only, variant=vid, fuse=2) -
                          untimed_ms([0] * LEVELS, variant=vid, fuse=2)) / ITERS[-1]
                 gbs = n0 * bpv / (it_ms / 1e3) / 1e9

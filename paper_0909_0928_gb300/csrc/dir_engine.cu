@@ -132,7 +132,8 @@ struct dir_ctx {
     char* img_pool = nullptr;
     char* A = nullptr;
     char* B = nullptr;
-    char* C = nullptr;     // Eqs. 3-6 split with the difference image: D of a level
+    char* C = nullptr;     // Eqs. 3-6 split with the difference image: D (and u) of a level;
+                           // Eq. 6's interleaved field
     size_t C_bytes = 0;
     double* red = nullptr;
     double* corr = nullptr;   // 4 sums per iteration of the correlation coefficient, or null
@@ -379,11 +380,11 @@ static void d_scratch(const dir_ctx* c, const Grid3& g, bool writes_u, dirk::For
 // Iteration schedule of pyramid level l: 0 force + smoothing kernels, 1 fused
 // iteration (the Gaussian of v_{k-1} folded into the force pass), 2 split
 // Gaussian (its x and y passes as their own kernel, its z pass inside the
-// force kernel), 3 split with the difference image (above).  All four give the
-// same field bit for bit.  fuse = 2 (the default) takes the split schedule
-// where it applies for Eqs. 1-2 on every level and for Eqs. 3-6 on the small
-// levels (there in form 3), otherwise the fused one on the small levels:
-// measured per level on the 256x256x100 pyramid.
+// force kernel), 3 split with the difference image, 4 resident in a cluster (both
+// above).  All five give the same field bit for bit.  fuse = 2 (the default) takes 4
+// on the small levels, else the split schedule where it applies (Eqs. 3-6: form 3,
+// or without room for D form 2 on levels of at most 2^21 voxels), otherwise the
+// fused one on the small levels: measured per level on the 256x256x100 pyramid.
 static int level_schedule(const dir_ctx* c, int l) {
     if (c->fp64 || c->p.plain_kernels) return 0;
     const Grid3& g = c->lv[l].g;
