@@ -140,7 +140,8 @@ typedef struct {
                                     force pass (Secs. 2.4, 3.3; dir_get_correlation); 0
                                     (default): not recorded */
     int pdl;                     /* 1 (default): on levels of 2^19 to 2^20 voxels without a stop
-                                    test (grouped batches: above 2^18 voxels per chunk), launch
+                                    test (grouped batches: above 2^18 voxels per chunk; without
+                                    a graph: up to 2^21 voxels), launch
                                     the iteration kernels as programmatic dependent launches
                                     (each starts its setup while the one before drains); 0:
                                     plain launches.  The same field either way */
