@@ -1977,7 +1977,7 @@ extern "C" int dir_register_noalloc(const float* static_img, const float* moving
     }
 
     // what is left holds the D scratch of Eqs. 3-6 and Eq. 6's interleaved field,
-    // as far as they fit (128x128x64, active, 200/100/50: 3.94 ms without, now 3.53)
+    // as far as they fit (128x128x64, active, 200/100/50: 3.94 -> 3.53 ms)
     const size_t offC = at;
     for (int l = 0; l < c.levels; ++l)
         if (p.iters[c.levels - 1 - l] > 0 && level_wants_d(&c, l))
