@@ -135,19 +135,19 @@ static cudaError_t launch_gzs_types(int variant, const ForceArgs& a, const Taps&
     }
 }
 
-// Brick depth.  Large levels: Eq. 1 takes 6 planes (four blocks per SM, as at 4,
-// with less halo), Eq. 2 with its M box 4 (6 and 8 leave three blocks per SM).
-// Below 16 six-plane bricks per SM: 4 planes while those number two per SM, else
-// 2; but where four-plane bricks are just over one wave of resident blocks, the
-// shallowest brick that makes it one wave.  Measured per iteration at depths
-// 2 / 4 / 6 / 8, Eq. 1 and Eq. 2:
-//   256x256x100  86.7 / 73.4 / 73.0 / 80.0 us    91.2 / 76.0 / 85.7 / 89.2
-//   193x171x87   48.4 / 41.7 / 42.1 / 44.9       51.0 / 43.2 / 48.5 / 49.9
-//   128x128x64   17.7 / 16.4 / 17.2 / 18.1       18.6 / 17.0 / 19.3 / 20.8
-//   128x128x50   15.6 / 14.8 / 14.2 / 14.4       15.8 / 16.9 / 18.6 / 15.8
-//   96x96x48     11.5 / 10.4 / 10.7 / 11.6       12.1 / 11.1 / 11.6 / 13.3
-//   96x96x24      7.2 /  7.8 /  8.0 /  8.6        7.6 /  8.2 /  8.7 / 10.3
-//   48x48x24      5.5 /  6.3 /  7.2 /  7.8 (1: 5.7)
+// Brick depth: 4 planes while those bricks number two per SM (four blocks per SM;
+// 6 and 8 spill, and with Eq. 2's M box leave three), else 2; but where four-plane
+// bricks are just over one wave of resident blocks, the shallowest brick that makes
+// it one wave.  Measured per iteration at depths 2 / 4 / 6 / 8, Eq. 1 and Eq. 2:
+//   512x512x160   531 /  439 /  479 /  522 us     557 /  468 /  520 /  537
+//   256x256x100  87.7 / 72.1 / 78.1 / 86.5       91.8 / 76.8 / 84.9 / 90.8
+//   193x171x87   49.2 / 41.0 / 44.8 / 49.1       51.7 / 44.1 / 48.4 / 51.7
+//   128x128x64   18.0 / 16.1 / 18.1 / 20.8       19.0 / 17.4 / 18.9 / 21.3
+//   128x128x50   16.0 / 14.7 / 14.8 / 15.4       16.0 / 17.4 / 18.6 / 16.1
+//   96x96x48     11.6 / 10.3 / 11.3 / 12.7       12.3 / 11.2 / 11.6 / 13.6
+//   96x96x24      7.4 /  7.6 /  8.5 /  9.2        7.8 /  8.3 /  8.6 / 10.5
+//   48x48x24      5.5 /  6.0 /  7.6 /  8.2        5.8 /  6.6 /  7.8 /  9.7
+// (int16 images: 512x512x160 541 / 432 / 453 / 454, 256x256x100 89 / 72 / 74 / 77)
 int force_zs_depth(int variant, const Grid3& g, int num_sms) {
     const long long bxy = (long long)((g.nx + FTX - 1) / FTX) * ((g.ny + FTY - 1) / FTY);
     return force_zs_depth_of(variant, num_sms, [&](int d) { return bxy * ((g.nz + d - 1) / d); });

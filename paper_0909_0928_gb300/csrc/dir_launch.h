@@ -105,7 +105,6 @@ int force_zs_depth(int variant, const Grid3& g, int num_sms);
 // its rule on any count of bricks by depth (Eqs. 1-2; a group of volumes)
 template <typename Bricks>
 int force_zs_depth_of(int variant, int num_sms, Bricks&& bricks) {
-    if (bricks(6) >= 16LL * num_sms) return variant == 0 ? 6 : 4;
     if (bricks(4) < 2LL * num_sms) return 2;
     const long long wave = 4LL * num_sms;  // resident four-plane bricks
     if (bricks(4) > wave && 2 * bricks(4) < 3 * wave)

@@ -55,9 +55,13 @@ __device__ __forceinline__ f32x2 f2_neg(f32x2 a) { return f2_pack(-f2_lo(a), -f2
 __device__ __forceinline__ f32x2 f2_sq3(f32x2 x, f32x2 y, f32x2 z) {
     return f2_fma(z, z, f2_fma(y, y, f2_mul(x, x)));
 }
-// |grad M| of Eq. (2): x x + y y + z z as the compiler contracts it, y y rounded
+// x x + y y + z z as the compiler contracts it in the scalar kernels: y y rounded
+__device__ __forceinline__ f32x2 f2_sq3_yxz(f32x2 x, f32x2 y, f32x2 z) {
+    return f2_fma(z, z, f2_fma(x, x, f2_mul(y, y)));
+}
+// |grad M| of Eq. (2)
 __device__ __forceinline__ f32x2 f2_norm_yxz(f32x2 x, f32x2 y, f32x2 z) {
-    const f32x2 s = f2_fma(z, z, f2_fma(x, x, f2_mul(y, y)));
+    const f32x2 s = f2_sq3_yxz(x, y, z);
     return f2_pack(r_sqrt(f2_lo(s)), r_sqrt(f2_hi(s)));
 }
 
@@ -224,32 +228,27 @@ __device__ __forceinline__ void pair_update(f32x2 d, const f32x2 (&gs)[3], const
     }
 }
 
-// Euclidean norm from its square, for the reductions: 0 for NaN, as
-// r_norm_fast (the larger of NaN and 0 is 0)
-__device__ __forceinline__ float norm_of_sq(float s) {
-    float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(s, 0.0f)));
-    return r;
-}
-
-// The reductions of one thread: sum d^2, sum |du|, sum |u| over its voxels
+// The reductions of one thread: sum d^2, sum |du|, sum |u| over its voxels.  The
+// norms are the scalar kernels' (r_norm_fast): not a number where the square
+// overflows, so that no stop test takes it for convergence, and right for
+// subnormal squares.
 struct PairSums {
     float d2 = 0.0f, du = 0.0f, u = 0.0f;
     __device__ __forceinline__ void add(f32x2 d, const f32x2 (&dr)[3], const f32x2 (&uu)[3], bool va,
                                         bool vb) {
         float da, db, wa, wb, sa, sb;
         f2_unpack(d, da, db);
-        f2_unpack(f2_sq3(dr[0], dr[1], dr[2]), wa, wb);
-        f2_unpack(f2_sq3(uu[0], uu[1], uu[2]), sa, sb);
+        f2_unpack(f2_sq3_yxz(dr[0], dr[1], dr[2]), wa, wb);
+        f2_unpack(f2_sq3_yxz(uu[0], uu[1], uu[2]), sa, sb);
         if (va) {
             d2 = fmaf(da, da, d2);
-            du += norm_of_sq(wa);
-            u += norm_of_sq(sa);
+            du += r_norm_fast(wa);
+            u += r_norm_fast(sa);
         }
         if (vb) {
             d2 = fmaf(db, db, d2);
-            du += norm_of_sq(wb);
-            u += norm_of_sq(sb);
+            du += r_norm_fast(wb);
+            u += r_norm_fast(sb);
         }
     }
 };

@@ -1,0 +1,65 @@
+"""The sums of an iteration (dir_get_history) and the stop test that reads them,
+where rounding or the ends of the float range show: what the plain-load kernels
+report, whichever kernels a level runs.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+# default: a resident level; fuse 4: the split kernels
+FORMS = {"resident": {}, "split": {"fuse": 4}}
+
+
+@pytest.fixture(scope="module")
+def dl():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_0909_0928_gb300 as dl
+    return dl
+
+
+def _register(dl, S, M, variant, n, start=None, **kw):
+    u0 = None if start is None else torch.tensor(np.ascontiguousarray(start)).cuda()
+    p = dl.dir_params_default(levels=1, iters=[n], alpha=0.7, init_field=u0, **kw)
+    ctx = dl.dir_create(S, M, S.shape[::-1], (1.0, 1.0, 1.0), dl.DIR_F32, False, variant, p)
+    try:
+        st = dl.dir_register(ctx)
+        return st.iters_run[0], dl.dir_get_history(ctx, n)
+    finally:
+        dl.dir_destroy(ctx)
+
+
+@pytest.mark.parametrize("form", list(FORMS))
+@pytest.mark.parametrize("value", [1e25, 1e19, 3.7, 0.1, 1e-3, 1e-18, 1e-20, 1e-21, 1e-24, 0.0,
+                                   np.inf, np.nan], ids=str)
+def test_norms_of_one_voxel(dl, value, form):
+    """A sum over one voxel is that voxel's norm, so it has to be the plain
+    kernels' bit for bit: squares that overflow (not a number, so that no stop
+    test takes them for convergence), that are subnormal, that underflow."""
+    S = np.full((1, 1, 1), 20.0, np.float32)
+    M = np.full((1, 1, 1), 21.0, np.float32)
+    u0 = np.float32(value) * np.array([1.0, -0.3, 0.7], np.float32).reshape(3, 1, 1, 1)
+    for variant in (0, 1, 2, 5):
+        want = _register(dl, S, M, variant, 3, u0, plain_kernels=1)[1]
+        got = _register(dl, S, M, variant, 3, u0, **FORMS[form])[1]
+        np.testing.assert_array_equal(got, want, err_msg=f"variant {variant}")
+
+
+@pytest.mark.parametrize("dims", [(8, 8, 4), (40, 32, 24), (129, 128, 60)],
+                         ids=["small", "tiles", "strips"])
+@pytest.mark.parametrize("value", [1e25, 1e-20], ids=str)
+def test_stop_test_at_the_ends_of_the_float_range(dl, dims, value):
+    """Equal constant images move nothing, so every norm of the start field is
+    met by every iteration: |u|^2 beyond the float range is no convergence and a
+    subnormal one is a norm like any other."""
+    S = np.full(dims[::-1], 20.0, np.float32)
+    u0 = np.full((3,) + dims[::-1], value, np.float32)
+    kw = dict(stop_mode=1, eps=1e-6, stop_window=3)
+    want = _register(dl, S, S, 0, 9, u0, plain_kernels=1, **kw)
+    got = _register(dl, S, S, 0, 9, u0, **kw)
+    assert want[0] == (9 if value > 1.0 else 4)
+    assert got[0] == want[0]
+    assert np.array_equal(np.isnan(got[1]), np.isnan(want[1]))
