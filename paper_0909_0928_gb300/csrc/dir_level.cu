@@ -340,32 +340,47 @@ __global__ void __launch_bounds__(LNT, 1) level_kernel(const __grid_constant__ L
     };
 
     // The sums of an iteration: every thread leaves its own in shared memory, and
-    // the last warp, which has the fewest tasks, adds them up during the x pass
-    // (FP32 over 64 threads, 8 lanes per sum) and the y pass (FP64 over the 8
-    // lanes) of the next iteration.
+    // the last three warps, which have the fewest tasks, add up one sum each during
+    // the x pass (a lane those of 16 threads) and the y pass (over the lanes) of the
+    // next iteration, FP64 across CTAs.  What an addition rounds away is kept beside
+    // the sum (Knuth's TwoSum; FP64 runs at 1/64 of the rate): beyond a thread
+    // nothing is lost to FP32, whose plain additions over 64 threads doubled the
+    // error of the sums (sum d^2 at 32x32x16 against 64 bits: 3.5e-9, 1.8e-9 in the
+    // split kernels, now 1.1e-9).
     float* const part = sm + L.off_p;
-    const bool adds_up = tid >= LNT - 32 && (tid & 31) < 24;
-    float part_sum = 0.0f;
+    const int lane = tid & 31, sum_of = (tid >> 5) - (LNT / 32 - 3);  // 0 .. 2, else negative
+    float sum_hi = 0.0f, sum_lo = 0.0f;
+    auto add = [&](float v) {
+        const float t = __fadd_rn(sum_hi, v), b = __fsub_rn(t, sum_hi);
+        sum_lo += __fadd_rn(__fsub_rn(sum_hi, __fsub_rn(t, b)), __fsub_rn(v, b));
+        sum_hi = t;
+    };
     auto reduce_threads = [&]() {
-        if (!adds_up) return;
-        const int k = (tid & 31) >> 3, j = tid & 7;
-        float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (sum_of < 0) return;
+        const float4* p = reinterpret_cast<const float4*>(part + sum_of * LNT) + lane;
+        sum_hi = sum_lo = 0.0f;
 #pragma unroll
-        for (int q = 0; q < LNT; q += 32) {
-            const float4 p = *reinterpret_cast<const float4*>(part + k * LNT + q + 4 * j);
-            f.x += p.x;
-            f.y += p.y;
-            f.z += p.z;
-            f.w += p.w;
+        for (int q = 0; q < LNT / 128; ++q) {
+            const float4 v = p[32 * q];
+            add(v.x);
+            add(v.y);
+            add(v.z);
+            add(v.w);
         }
-        part_sum = (f.x + f.y) + (f.z + f.w);
     };
     auto reduce_lanes = [&](int it) {
-        if (!adds_up) return;
-        double d = (double)part_sum;
+        if (sum_of < 0) return;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0x00ffffffu, d, o);
-        if ((tid & 7) == 0) atomicAdd(a.red + 3 * it + ((tid & 31) >> 3), d);
+        for (int o = 16; o > 0; o >>= 1) {
+            const float hi = __shfl_down_sync(0xffffffffu, sum_hi, o);
+            const float lo = __shfl_down_sync(0xffffffffu, sum_lo, o);
+            add(hi);
+            sum_lo += lo;
+        }
+        // an infinite sum leaves infinity - infinity in what was rounded away
+        if (lane == 0)
+            atomicAdd(a.red + 3 * it + sum_of,
+                      isfinite(sum_hi) ? (double)sum_hi + (double)sum_lo : (double)sum_hi);
     };
 
     for (int it = 0; it < a.iters; ++it) {

@@ -63,3 +63,34 @@ def test_stop_test_at_the_ends_of_the_float_range(dl, dims, value):
     assert want[0] == (9 if value > 1.0 else 4)
     assert got[0] == want[0]
     assert np.array_equal(np.isnan(got[1]), np.isnan(want[1]))
+
+
+@pytest.mark.parametrize("dims", [(32, 32, 16), (16, 16, 8), (25, 25, 10)],
+                         ids=lambda d: "x".join(map(str, d)))
+def test_sum_of_one_large_and_many_small_terms(dl, dims):
+    """d = 1 everywhere but 2^15 in one voxel: an FP32 sum that holds 2^30 loses
+    every 1 added to it.  The sum of a resident level may lose no more of them than
+    the plain kernels', whose FP32 sums end with a warp."""
+    n = dims[0] * dims[1] * dims[2]
+    exact = float(n - 1) + 2.0 ** 30
+    for at in (0, n // 3, n // 2 + 17, n - 1):
+        S = np.zeros(dims[::-1], np.float32)
+        M = np.ones(dims[::-1], np.float32)
+        M.reshape(-1)[at] = 2.0 ** 15
+        for variant in (0, 2, 5):
+            plain = _register(dl, S, M, variant, 1, plain_kernels=1)[1][0, 0] * n
+            level = _register(dl, S, M, variant, 1)[1][0, 0] * n
+            assert abs(level - exact) <= abs(plain - exact), (at, variant, exact - plain)
+
+
+def test_infinite_sum_of_a_resident_level(dl):
+    """One difference whose square overflows makes the sum infinite, as in the
+    plain kernels, not NaN."""
+    S = np.zeros((8, 16, 16), np.float32)
+    M = np.ones_like(S)
+    M[3, 4, 5] = 1e25
+    for variant in (0, 2, 5):
+        plain = _register(dl, S, M, variant, 1, plain_kernels=1)[1]
+        level = _register(dl, S, M, variant, 1)[1]
+        np.testing.assert_array_equal(level[:, 0], plain[:, 0])
+        assert np.isinf(plain[0, 0])
