@@ -94,3 +94,28 @@ def test_infinite_sum_of_a_resident_level(dl):
         level = _register(dl, S, M, variant, 1)[1]
         np.testing.assert_array_equal(level[:, 0], plain[:, 0])
         assert np.isinf(plain[0, 0])
+
+
+@pytest.mark.parametrize("form", list(FORMS))
+@pytest.mark.parametrize("dims", [(32, 32, 16), (16, 16, 8), (25, 25, 10)],
+                         ids=lambda d: "x".join(map(str, d)))
+def test_correlation_beside_one_large_term(dl, dims, form):
+    """S and M are 1 but for a voxel where S is L, M 0 and another where it is the
+    other way round, so that the covariance is what the L^2 in sum S^2 leaves of the
+    ones beside it: an FP32 sum of at most 32 voxels loses at most 31 of them."""
+    n = dims[0] * dims[1] * dims[2]
+    large = 2.0 ** 15
+    for at in (5, n // 3):
+        S = np.ones(dims[::-1], np.float32)
+        M = np.ones(dims[::-1], np.float32)
+        S.reshape(-1)[at], M.reshape(-1)[at] = large, 0.0
+        S.reshape(-1)[at + n // 2], M.reshape(-1)[at + n // 2] = 0.0, large
+        exact = np.corrcoef(S.ravel().astype(np.float64), M.ravel().astype(np.float64))[0, 1]
+        for variant in (0, 2, 5):
+            p = dl.dir_params_default(levels=1, iters=[1], alpha=0.7, correlation=1,
+                                      **FORMS[form])
+            ctx = dl.dir_create(S, M, dims, (1.0, 1.0, 1.0), dl.DIR_F32, False, variant, p)
+            dl.dir_register(ctx)
+            rho = dl.dir_get_correlation(ctx, 1)[0]
+            dl.dir_destroy(ctx)
+            assert abs(rho - exact) <= 32.0 / (n * float(S.var(dtype=np.float64))), (variant, at)
