@@ -2027,7 +2027,20 @@ extern "C" int dir_register_noalloc(const float* static_img, const float* moving
     c.ctl = reinterpret_cast<int*>(base + offCtl);
     c.derr = reinterpret_cast<int*>(base + offErr);
 
-    int rc = upload_pair(&c, static_img, moving_img, 1, c.stream);
+    // On an x axis of one voxel the gathers read the row padding beside it with
+    // weight 0: zero in the images of such levels (the coarsest), which dir_create
+    // clears once, whatever an earlier call left there
+    int rc = DIR_OK;
+    for (int l = 0; l < c.levels; ++l) {
+        if (c.lv[l].g.nx > 1) continue;
+        e = cudaMemsetAsync(c.lv[l].S, 0, offA - lvl_off[l][0], c.stream);
+        if (e != cudaSuccess) {
+            set_err(&c, "cudaMemsetAsync", e);
+            rc = DIR_ECUDA;
+        }
+        break;
+    }
+    if (rc == DIR_OK) rc = upload_pair(&c, static_img, moving_img, 1, c.stream);
     if (rc == DIR_OK) rc = enqueue_registration(&c, c.stream, false);
     if (rc == DIR_OK && dirk::launch_export_field(c.fp64, c.field_type, c.final_field, c.lv[0].g,
                                                   1.0, 1.0, 1.0, field_out, false,

@@ -42,8 +42,8 @@ constexpr int HX = FTX + 2, HY = FTY + 2;
 // software trilinear, clamped): the upper corner is one element to the right
 // along x and sy / sz elements further along y / z, with sy or sz 0 on an axis
 // of one voxel.  On an x axis of one voxel the weight of the right neighbour is
-// 0 and that neighbour is row padding (zero in the image pool), so the read is
-// harmless.
+// 0 and that neighbour is row padding, zero in the images of a level (dir_create
+// and dir_register_noalloc clear it), so the read is harmless.
 struct Interp {
     int nx1, ny1, nz1;     // n - 1
     int nxm2, nym2, nzm2;  // max(n - 2, 0): largest lower corner
