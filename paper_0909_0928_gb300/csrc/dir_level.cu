@@ -34,6 +34,7 @@
 #include <algorithm>
 
 #include "dir_launch.h"
+#include "dir_once.h"
 #include "dir_pair.cuh"
 #include "dir_stencil.cuh"
 
@@ -548,16 +549,10 @@ struct ActiveClusters {
     int n[kLevelCluster + 1];
 };
 const ActiveClusters* active_clusters() {
-    static std::atomic<int> known[KernelSetup::kMaxDevices];  // 0 unknown, 1 no, 2 yes
-    static ActiveClusters table[KernelSetup::kMaxDevices];
-    static std::mutex mutex;
+    static OncePerDevice<ActiveClusters, KernelSetup::kMaxDevices> table;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= KernelSetup::kMaxDevices)
-        return nullptr;
-    int k = known[dev].load(std::memory_order_acquire);
-    if (k == 0) {
-        std::lock_guard<std::mutex> lock(mutex);
-        ActiveClusters& t = table[dev];
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    const ActiveClusters* t = table.get(dev, [](ActiveClusters& t) {
         const bool ok = setup_level<0, float>() == cudaSuccess;
         for (int C = 1; C <= kLevelCluster; ++C) {
             cudaLaunchConfig_t cfg = {};
@@ -577,10 +572,8 @@ const ActiveClusters* active_clusters() {
             t.n[C] = n;
         }
         cudaGetLastError();
-        k = t.n[kLevelCluster / 2] > 0 ? 2 : 1;
-        known[dev].store(k, std::memory_order_release);
-    }
-    return k == 2 ? &table[dev] : nullptr;
+    });
+    return t && t->n[kLevelCluster / 2] > 0 ? t : nullptr;
 }
 
 template <int V, typename TI>
