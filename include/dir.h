@@ -311,11 +311,14 @@ void dir_batch_destroy(dir_batch* batch);  /* NULL-safe */
  * Launch-shape autotuning for one context, after a finished dir_register:
  * for each pyramid level, times the force kernel with 1, 2, 4 and 8 voxels
  * per thread along z and the smoothing kernel with several z chunks (on
- * levels of the split schedule, the z + force kernel and the x/y kernel)
+ * levels of the split schedule, the z + force kernel, also with 6, and the x/y
+ * kernel, whose z chunk is a strip's length in boxes of seven rows where it
+ * runs strips; above 2^20 voxels the two kernels of Eqs. (3)-(6) with 4 and 8)
  * (`reps` launches each), keeps the fastest of each for the context's later
- * registrations (and batches built afterwards), and writes them to
+ * registrations (and batches on branches built afterwards), and writes them to
  * shapes_out[2*l], shapes_out[2*l+1] for level l (finest = 0) if not NULL.
- * The registered field is kept.
+ * A level that runs in one launch (schedule 4) has no shape to choose and
+ * reports 2, 0.  The registered field is kept.
  */
 int dir_autotune(dir_ctx* ctx, int reps, int* shapes_out);
 

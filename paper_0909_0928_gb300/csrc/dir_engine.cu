@@ -145,7 +145,8 @@ struct dir_ctx {
     int fused_level[DIR_MAX_LEVELS];
     int tune_depth[DIR_MAX_LEVELS] = {0};    // force brick depth per level, 0 = heuristic
     int tune_zchunk[DIR_MAX_LEVELS] = {0};   // smoothing z chunk per level (of the x/y kernel
-                                             // on split levels), 0 = the launcher's choice
+                                             // on split levels, or boxes of its strips),
+                                             // 0 = the launcher's choice
     char* final_field = nullptr;
     bool have_field = false;
     bool pending = false;
@@ -725,6 +726,7 @@ static int enqueue_registration(dir_ctx* c, cudaStream_t s, bool capturing) {
             }
             sa.in = vbuf;
             sa.out = tbuf;
+            sa.zchunk = 0;           // the tuned one is the x/y kernel's
             sa.iter = 0;
             sa.stop_iter = nullptr;  // always: v of the last iteration run
             CK(c, dirk::launch_smooth(f64, sa, c->num_sms, s, plain));
@@ -1570,6 +1572,7 @@ static int enqueue_grouped_chunk(dir_ctx* const* ctxs, const std::vector<int>& j
             dirk::SmoothArgs sa = level_smooth_args(c, lc);
             sa.in = oth[q];
             sa.out = cur[q];
+            sa.zchunk = 0;  // the tuned one is the x/y kernel's
             sa.stop_iter = nullptr;
             sa.iter = 0;
             CK(c, dirk::launch_smooth(false, sa, c->num_sms, lanes.of(q), false));
@@ -1801,16 +1804,27 @@ extern "C" int dir_autotune(dir_ctx* c, int reps, int* shapes_out) {
         fa.err = c->derr;
         fa.pf_stride = c->num_sms;  // as in the registration
         const int sched = level_schedule(c, l);  // time the kernels the level runs
+        if (sched == 4) {  // in one launch without a shape to choose
+            if (shapes_out) {
+                shapes_out[2 * l] = 2;  // its threads take voxels in pairs along z
+                shapes_out[2 * l + 1] = 0;
+            }
+            continue;
+        }
         const bool split = sched >= 2;
         float best = 1e30f;
         int best_d = 0;
-        const int depths[5] = {1, 2, 4, 8, 6};  // 6: the split force kernel only
-        // schedule 3: the z + D and stencil force kernels, D in the scratch
+        const int depths[5] = {1, 2, 4, 8, 6};
+        int first = 0;
+        const int last = sched == 2 ? 5 : 4;  // 6: the z + force kernel only
+        // schedule 3: the z + D and stencil force kernels, D in the scratch; without
+        // u there they are 4 deep at least
         dirk::ForceArgs za = fa, ta = fa;
         if (sched == 3) {
             d_scratch(c, g, level_writes_u(c, l), za, ta);
+            if (!level_writes_u(c, l)) first = 2;
         }
-        for (int di = 0; di < (sched == 2 ? 5 : 4) && rc == DIR_OK; ++di) {
+        for (int di = first; di < last && rc == DIR_OK; ++di) {
             const int d = depths[di];
             fa.depth = ta.depth = d;
             za.depth = std::min(d, kZdMaxDepth);
@@ -1840,8 +1854,11 @@ extern "C" int dir_autotune(dir_ctx* c, int reps, int* shapes_out) {
         int best_z = 0;
         int cand[16], nc = 0;
         cand[nc++] = 0;  // one wave (the default)
-        for (int z = 1; z < g.nz && nc < 15; z *= 2) cand[nc++] = z;
-        cand[nc++] = g.nz;
+        // planes per block, or boxes per strip of the x/y kernel (2 at least)
+        const int strip = split ? dirk::smooth_xy_longest_strip(g, c->num_sms) : 0;
+        const int most = strip ? strip : g.nz;
+        for (int z = strip ? 2 : 1; z < most && nc < 15; z *= 2) cand[nc++] = z;
+        cand[nc++] = most;
         for (int k = 0; k < nc && rc == DIR_OK; ++k) {
             sa.zchunk = cand[k];
             float ms = 0.0f;

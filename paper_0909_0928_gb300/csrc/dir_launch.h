@@ -95,6 +95,9 @@ bool smooth_xy_supported(const SmoothArgs& a);
 // is then not read)
 cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s,
                              const StopTest& test = StopTest());
+// 0 where it runs tiles (a.zchunk: planes per block), else the boxes of a strip as
+// long as the volume (a.zchunk: boxes per strip, 2 up to that)
+int smooth_xy_longest_strip(const Grid3& g, int num_sms);
 
 // Force pass of Eqs. 1-2 whose u is G_z * t, t = a.u the output of
 // launch_smooth_xy (single-precision field, float or int16 images, radius 3):

@@ -442,6 +442,8 @@ static cudaError_t launch_sxy(const SmoothArgs& a, int num_sms, const StopTest& 
                      test);
 }
 
+constexpr int kMaxStripBoxes = 64;  // of a strip whose length the caller chose
+
 static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, const StopTest& test,
                                     cudaStream_t s) {
     CUtensorMap map;
@@ -451,7 +453,7 @@ static cudaError_t launch_xy_strips(const SmoothArgs& a, int num_sms, const Stop
     const cudaError_t e =
         setup_kernel(setup, smooth_xy_strip_kernel, XYSMEM, 32 * XYWARPS, &per_sm);
     if (e != cudaSuccess) return e;
-    const int nb = a.zchunk > 0 ? std::max(2, std::min(a.zchunk, 64))
+    const int nb = a.zchunk > 0 ? std::max(2, std::min(a.zchunk, kMaxStripBoxes))
                                 : xy_strip_boxes(&a.g, 1, per_sm * num_sms * XYWARPS);
     const XYStrips st = xy_strips(a.g, nb);
     return launch_ex(smooth_xy_strip_kernel, dim3((unsigned)st.blocks()), dim3(32 * XYWARPS, 1, 1),
@@ -493,6 +495,11 @@ static cudaError_t launch_types(const SmoothArgs& a, int num_sms, cudaStream_t s
 
 bool smooth_xy_supported(const SmoothArgs& a) {
     return a.ncomp == 3 && a.in_type == kStoreF32 && a.out_type == kStoreF32 && a.taps.R == XYR;
+}
+
+int smooth_xy_longest_strip(const Grid3& g, int num_sms) {
+    if (!xy_use_strips(&g, 1, num_sms)) return 0;
+    return std::max(2, std::min((g.ny + 2 * XYR + XYB - 1) / XYB, kMaxStripBoxes));
 }
 
 cudaError_t launch_smooth_xy(const SmoothArgs& a, int num_sms, cudaStream_t s,
