@@ -141,7 +141,7 @@ typedef struct {
                                     (default): not recorded */
     int pdl;                     /* 1 (default): on levels of 2^19 to 2^20 voxels without a stop
                                     test (grouped batches: above 2^18 voxels per chunk; without
-                                    a graph: up to 2^21 voxels), launch
+                                    a graph: of any size), launch
                                     the iteration kernels as programmatic dependent launches
                                     (each starts its setup while the one before drains); 0:
                                     plain launches.  The same field either way */

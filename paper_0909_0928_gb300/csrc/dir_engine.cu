@@ -294,16 +294,17 @@ static int record(dir_ctx* c, cudaEvent_t e, cudaStream_t s, bool capturing) {
 // 193x171x87 45.85 -> 46.74 / 59.63 -> 61.32, 256x256x100 72.98 -> 75.43 /
 // 106.97 -> 107.25 (Eq. 6 124.98 -> 127.76).
 // Those are graph nodes, 0.7 us apart; two kernels launched directly are 2 to 4 us
-// apart, which the early start hides on every level up to 2^21 voxels: 40x32x16
-// 10.4 -> 6.1 / 12.5 -> 8.0, 97x63x48 16.5 -> 11.7 / 20.6 -> 14.3, 160x100x80
-// 24.7 -> 20.5 / 33.0 -> 26.3 (dir_register_noalloc).
+// apart, which the early start hides on levels of any size (passive / active):
+// 40x32x16 10.4 -> 6.1 / 12.5 -> 8.0, 97x63x48 16.5 -> 11.5 / 20.5 -> 14.4,
+// 128x128x128 30.8 -> 26.1 / 41.1 -> 34.4, 193x171x87 46.3 -> 42.6 / 60.8 -> 58.5,
+// 256x256x100 77.7 -> 72.5 / 105.8 -> 100.7 (Eq. 6 122.8 -> 118.1).
 // Not with a stop test (the kernels read the stop flag before they wait), nor
 // with timing events between the kernels. Split schedule only: the same
 // launches made the force + smoothing kernels slower.
 static bool level_pdl(const dir_ctx* c, const Grid3& g, bool timed, bool capturing) {
     const long long n = (long long)g.nx * g.ny * g.nz;
     return c->p.pdl && c->p.stop_mode == 0 && !timed && !c->fp64 && !c->p.plain_kernels &&
-           (capturing ? n >= (1LL << 19) && n <= (1LL << 20) : n <= (1LL << 21));
+           (!capturing || (n >= (1LL << 19) && n <= (1LL << 20)));
 }
 
 // The split kernels: FP32 field, float or int16 images, radius 3

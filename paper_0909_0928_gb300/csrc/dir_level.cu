@@ -615,8 +615,12 @@ cudaError_t launch_level_types(int variant, const LevelGroup& G, int smem, cudaS
 // 32x32x16 16: 3.83 / 4.3, 8: 5.9 / 6.0, 6: 7.7 / 7.3), and clusters that do not
 // run at once take turns.  A GB300 holds 7 clusters of 16 CTAs, 15 of 8, 23 of 6:
 // 16 levels of 32x32x16 took 11.8 us an iteration in two turns of 8 CTAs and
-// take 7.8 in one of 6 (the grouped split kernels: 10.4); 8 levels of 16x16x8
-// 5.3 us in two turns of 16, now 2.5 in one of 8.
+// take 7.9 in one of 6 (the grouped split kernels: 10.4); 8 levels of 16x16x8
+// 5.3 us in two turns of 16, now 2.5 in one of 8.  The same model serves the laws
+// with a third barrier: its choice is the fastest of 4 to 16 CTAs, or within 2 %
+// of it, for Eqs. 3 and 6 too (16x16x8 alone 8: 3.48 / 3.72 us, 16: 3.47 / 3.72;
+// 32x32x16 alone 16: 5.1 / 5.7, 12: 6.8 / 7.3; 16 of 25x25x10 6: 7.0 / 7.8, 12: 10.1
+// / 11.1; 16 of 32x32x16 6: 10.1, Eq. 6 12: 14.9, 8: 15.3 / 17.5).
 int level_cluster(int variant, const Grid3* g, int n) {
     const ActiveClusters* active = active_clusters();
     int best_c = kLevelCluster / 2;

@@ -94,15 +94,17 @@ def test_large_chunks(dl, sizes, variant, i16):
     _check_batch(dl, GROUPS[sizes], variant, i16, [3], ())
 
 
+@pytest.mark.parametrize("graph", [1, 0], ids=["graph", "direct"])
 @pytest.mark.parametrize("variant", [0, 1, 2, 5])
 @pytest.mark.parametrize("dims", [(193, 171, 87), (161, 149, 49), (129, 127, 61), (260, 50, 70)],
                          ids=lambda d: "x".join(map(str, d)))
-def test_strips_with_remainders(dl, dims, variant):
+def test_strips_with_remainders(dl, dims, variant, graph):
     pair = _pair(dims, 90, variant == 1)
-    ctx = _context(dl, pair, dims, variant, [3])
+    # launched directly the kernels start before the one before them has ended
+    ctx = _context(dl, pair, dims, variant, [6], use_graph=graph)
     try:
         dl.dir_register(ctx)
         got = _field(dl, ctx, dims)
     finally:
         dl.dir_destroy(ctx)
-    assert np.array_equal(got, _plain(dl, pair, dims, variant, [3]), equal_nan=True)
+    assert np.array_equal(got, _plain(dl, pair, dims, variant, [6]), equal_nan=True)
