@@ -223,10 +223,12 @@ __device__ __forceinline__ void block_reduce3_atomic(Real a, Real b, Real c, dou
 // The sums of the correlation coefficient of the warped image with its
 // reference (Secs. 2.4, 3.3): per voxel b (S; Eq. 6: the warped static image)
 // and d = W - b; the field's own statistics keep Sum d^2.  Accumulated per
-// thread, then over 8 lanes in the arithmetic type and beyond in double into
-// out[0..3] = {Sum b, Sum b^2, Sum d, Sum b d}.  Eight lanes, not a warp: the
+// thread, then over LANES lanes in the arithmetic type and beyond in double into
+// out[0..3] = {Sum b, Sum b^2, Sum d, Sum b d}.  Less than a warp: the
 // coefficient is a small difference of these sums, and a thread has up to eight
-// voxels of its own (error against 64 bits at 16x16x8 6.0e-9 with a warp's).
+// voxels of its own (error against 64 bits of resident 16x16x8 levels 6.0e-9 with a
+// warp's, 1.4e-9 with eight lanes').  Sixteen in blocks of 256: 256 bytes of shared
+// memory; 512 cost the deep stencil force kernel its fourth block per SM.
 template <typename Real>
 struct CorrSums {
     Real b = 0, bb = 0, d = 0, bd = 0;
@@ -238,20 +240,20 @@ struct CorrSums {
     }
 };
 
-template <int NT, typename Real>
+template <int NT, typename Real, int LANES = sizeof(Real) == 8 ? 32 : 16>
 __device__ __forceinline__ void block_reduce4_atomic(const CorrSums<Real>& s, double* out) {
     static_assert(NT % 32 == 0, "block size must be whole warps");
-    constexpr int NP = NT / 8;  // partial sums per value: 8 lanes each
+    constexpr int NP = NT / LANES;  // partial sums per value
     __shared__ Real red4_s[4][NP];
     Real v[4] = {s.b, s.bb, s.d, s.bd};
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
+    for (int o = LANES / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    if ((tid & 7) == 0)
+    if (tid % LANES == 0)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) red4_s[k][tid >> 3] = v[k];
+        for (int k = 0; k < 4; ++k) red4_s[k][tid / LANES] = v[k];
     __syncthreads();
     if (tid < 32) {
         double dv[4] = {0.0, 0.0, 0.0, 0.0};

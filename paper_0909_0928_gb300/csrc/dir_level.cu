@@ -22,8 +22,8 @@
 // theirs.  Only the level's starting and resulting field touch global memory.
 //
 // Measured per iteration, split kernels -> this, Eq. 1 / Eq. 3: 16x16x8 4.84 ->
-// 2.65 us / 6.5 -> 3.4, 25x25x10 4.9 -> 3.3 / 6.4 -> 4.4, 32x32x16 4.88 -> 3.82 /
-// 6.35 -> 4.96; 48x43x22 (45,000 voxels) is faster split, so levels above 16,384
+// 2.52 us / 6.5 -> 3.5, 25x25x10 4.9 -> 3.4 / 6.4 -> 4.4, 32x32x16 4.88 -> 3.92 /
+// 6.35 -> 5.1; 48x43x22 (45,000 voxels) is faster split, so levels above 16,384
 // voxels stay there.  What bounds it: a cluster barrier takes 0.5 us with the halo
 // stores before it (two per iteration, three for Eqs. 3-6), the rest is one
 // dependent chain per pass on a few warps per SM; at 32x32x16 the force itself
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(LNT, 1) level_kernel(const __grid_constant__ L
         part[tid] = sums.d2;
         part[LNT + tid] = sums.du;
         part[2 * LNT + tid] = sums.u;
-        if (a.corr) block_reduce4_atomic<LNT, float>(corr_s, a.corr + 4 * it);
+        if (a.corr) block_reduce4_atomic<LNT, float, 8>(corr_s, a.corr + 4 * it);
         cluster_barrier();
     }
     // the level's result: u = G v of the last iteration
