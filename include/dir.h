@@ -116,8 +116,11 @@ typedef struct {
                                     once more after the difference image: a z-pass kernel
                                     writes D = W - S once per voxel (Eq. 6: both warped
                                     differences) to a scratch of 1 (Eq. 6: 2) floats per voxel
-                                    of the level, and a stencil kernel forms the force from
+                                    of the level, on levels of at most 2^20 voxels u beside it
+                                    (3 more), and a stencil kernel forms the force from
                                     them, instead of interpolating W on every brick's halo.
+                                    (Eq. 6's output step takes 4 floats per voxel of the
+                                    finest level of the same scratch.)
                                     2 (default): as 4 where it applies, and on levels of at most
                                     16,384 voxels without a stop test or timing all iterations
                                     in one launch, the field in the shared memory of a
@@ -193,7 +196,8 @@ int dir_params_default(dir_params* p);
  *   params                  NULL for defaults
  *   cuda_stream             a cudaStream_t, or NULL for the legacy default stream
  * The context owns all device memory it allocates (sized for the finest level,
- * about 9 floats per voxel plus the pyramid).  Returns DIR_OK and sets *out, or
+ * about 9 floats per voxel plus the pyramid, and for Eqs. (3)-(6) the scratch that
+ * params.fuse names).  Returns DIR_OK and sets *out, or
  * an error and sets *out = NULL.
  */
 int dir_create(dir_ctx** out, const void* static_img, const void* moving_img, const int dims[3],
@@ -256,7 +260,8 @@ int dir_get_history(dir_ctx* ctx, double* out, int max_iters);
  * update, in the order run (coarsest level first): the similarity measure that
  * Sec. 2.4 contrasts with the relative norm and Sec. 3.3 (Fig. 3) plots
  * against the iterations.  Its sums are reduced on the device in the force
- * pass (FP32 within a block, FP64 across blocks); the quotient is formed here.
+ * pass (FP32 over the voxels of at most 16 threads, FP64 beyond); the quotient
+ * is formed here.
  * Writes min(max_iters, iterations run) values (NaN where an image is
  * constant) to the host array out and returns that count; DIR_EUNSUPPORTED
  * unless the context was created with correlation = 1 or stop_mode = 2,

@@ -285,14 +285,16 @@ static int record(dir_ctx* c, cudaEvent_t e, cudaStream_t s, bool capturing) {
 // Programmatic dependent launch of a level's iteration kernels, on levels of
 // 2^19 to 2^20 voxels: a kernel's blocks set up and copy the static images
 // while the one before drains its last wave (they start only once all its
-// blocks have). It pays where a kernel is one or two waves long. Measured per
-// iteration, plain -> dependent, passive / active: 128x128x40 14.66 -> 14.03 /
-// 17.98 -> 17.74 us, 128x128x50 14.84 -> 14.38 / 19.96 -> 19.59, 160x160x40
-// 18.24 -> 18.07 / 22.17 -> 21.27; below, 96x96x48 11.70 -> 12.29 / 14.08 ->
-// 15.56; above, where the early blocks only take memory and slots from the
-// kernel that still runs, 160x160x50 21.22 -> 23.48 / 24.64 -> 25.53,
-// 193x171x87 45.85 -> 46.74 / 59.63 -> 61.32, 256x256x100 72.98 -> 75.43 /
-// 106.97 -> 107.25 (Eq. 6 124.98 -> 127.76).
+// blocks have). It pays where a kernel is one or two waves long, and there by
+// little. Measured per iteration, plain -> dependent, Eq. 1 / Eq. 3 / Eq. 6:
+// 128x128x50 15.29 -> 14.83 / 18.96 -> 18.97 / 20.96 -> 20.76 us, 128x128x40 13.90
+// -> 14.49 / 17.83 -> 17.48 / 19.43 -> 19.02, 160x160x40 15.84 -> 16.31 / 20.85 ->
+// 21.21 / 22.59 -> 23.19; below, 96x96x48 10.44 -> 10.46 / 13.19 -> 12.91 / 14.22 ->
+// 14.30, 64x64x25 5.98 -> 6.60 / 8.12 -> 9.91 / 8.40 -> 10.18; above, where the
+// early blocks only take memory and slots from the kernel that still runs,
+// 160x160x50 19.40 -> 19.52 / 25.46 -> 26.84 / 28.79 -> 29.96, 193x171x87 41.16 ->
+// 41.84 / 53.76 -> 57.02 / 64.19 -> 67.73, 256x256x100 72.18 -> 71.96 / 97.46 ->
+// 99.47 / 113.6 -> 116.1.
 // Those are graph nodes, 0.7 us apart; two kernels launched directly are 2 to 4 us
 // apart, which the early start hides on levels of any size (passive / active):
 // 40x32x16 10.4 -> 6.1 / 12.5 -> 8.0, 97x63x48 16.5 -> 11.5 / 20.5 -> 14.4,

@@ -5,7 +5,8 @@
 // volumes (dir_grouped.cu).  Each call handles the block at BlockPos bp of its
 // own volume's grid.
 //
-// Launched with programmatic dependent launch (coarse levels, no stop test),
+// Launched with programmatic dependent launch (no stop test; level_pdl in the
+// engine has the levels),
 // a block starts while the kernel before still runs: it sets up its barriers
 // and copies the static images, then waits (pdl_wait) before it reads the
 // field the kernel before wrote or writes one that kernel reads.  The stop

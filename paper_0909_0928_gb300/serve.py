@@ -40,7 +40,7 @@ def footprint_bytes(dims, levels: int, elem: int = 4, field_elem: int | None = N
                     scratch_planes: int = 0) -> int:
     """Device bytes one context holds: pyramid images (2 per level, pitched
     rows), two fields of the finest size, scratch_planes more finest-size
-    float volumes (the D scratch of Eqs. 3-6), the staging buffer of the
+    float volumes (the D and u scratch of Eqs. 3-6), the staging buffer of the
     host field read-back (3 N floats), plus a margin for reduction rows and
     padding."""
     nx, ny, nz = dims
@@ -69,9 +69,10 @@ def request_footprint(req) -> int:
     p = req.params
     elem = 8 if p.precision == DIR_F64 else 4
     fe = 2 if p.field_dtype == DIR_BF16 else elem
-    # Eqs. 3-6 under the default schedule (and fuse = 4): D = W - S of the finest
-    # level (Eq. 6: both warped differences).  The context takes 1 (Eq. 6: 2)
-    # floats per voxel; admission keeps 4 (5), three of them headroom
+    # Eqs. 3-6 under the default schedule (and fuse = 4), floats per voxel of the
+    # finest level: 1 for D = W - S (Eq. 6: 2, both warped differences) and, on
+    # levels of at most 2^20 voxels, 3 for u; Eq. 6's output step takes 4 of them at
+    # any size.  So 4 (5) is what small volumes and Eq. 6 need, no headroom
     planes = 0
     if (req.variant >= 2 and p.precision != DIR_F64 and p.field_dtype != DIR_BF16
             and p.fuse in (2, 4) and not p.plain_kernels):
